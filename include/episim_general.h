@@ -165,21 +165,22 @@ sim_status gen_counters(gen_handle* h, int64_t* counters);
  *       as a CUDA graph (captured once per (first day, ndays));
  *   GEN_OPT_WARP_THRESHOLD: nodes whose initial population (sum of u0) is at least
  *       this run the stochastic step one per warp, 32 draws at a time with a
- *       fixed-point iteration over the lanes (-1: automatic, 600);
+ *       fixed-point iteration over the lanes (-1: automatic, the largest nodes, as
+ *       many as leave each unit of work a resident warp, and those from 600 on);
  *   GEN_OPT_GROUP_THRESHOLD: nodes below the warp threshold whose initial
  *       population is at least this run four per warp, 8 lanes and 8 draws at a
- *       time each (-1: automatic, 150); the rest one per thread;
+ *       time each (-1: automatic, 300); the rest one per thread;
  *   GEN_OPT_CLOCK_MARGIN: k in [0, 16].  Every node-day (one per thread, per
  *       warp or per 8-lane segment) first runs with binary32 rates and partial
- *       sums and a binary32 clock accumulated in fixed point, whose distance to
- *       the binary64 clock of Eq. (numstep3) is bounded below 2^-16 of a day
- *       (product-form rates of at most 32 transitions, constants and continuous
- *       variables within [2^-30, 2^30], populations below 2^21; other node-days
- *       run exactly); a selection is taken in binary32 only when decisive (Eq.
- *       (sampling2), else binary64), and a stop/continue decision within 2^-k of
- *       the day's end reruns the node-day with the binary64 arithmetic.  k = 16
- *       (default) is the tightest safe margin; smaller k only reruns more
- *       node-days; 0 runs every node-day exactly. */
+ *       sums and a binary32 clock whose distance to the binary64 clock of Eq.
+ *       (numstep3) is bounded below 2^-16 of a day (product-form rates of at most
+ *       32 transitions, k_j y_q below 2^60, populations below 2^21; other
+ *       node-days run exactly); a selection is taken in binary32 only when
+ *       decisive (Eq. (sampling2), else binary64), and a stop/continue decision
+ *       within the margin of the day's end reruns the node-day with the binary64
+ *       arithmetic.  k = 16 (default) is the method's own bound, below 2^-16;
+ *       smaller k, a margin of 2^-k, only reruns more node-days; 0 runs every
+ *       node-day exactly. */
 enum { GEN_OPT_LAUNCH = 1, GEN_OPT_WARP_THRESHOLD = 2, GEN_OPT_GROUP_THRESHOLD = 3, GEN_OPT_CLOCK_MARGIN = 4 };
 sim_status gen_set_option(gen_handle* h, int32_t option, int64_t value);
 

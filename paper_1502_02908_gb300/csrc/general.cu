@@ -63,7 +63,10 @@ __device__ __forceinline__ double gen_y_next(const GenModelDev& m, const GenRepP
   const double omb = __dsub_rn(1.0, p.beta[q][season_of(day)]);
   double mid;
   if (m.den[q] == 0u) mid = __dmul_rn(p.alpha[q], U);
-  else mid = D > 0.0 ? __ddiv_rn(__dmul_rn(p.alpha[q], U), D) : 0.0;
+  else {
+    const double aU = __dmul_rn(p.alpha[q], U);
+    mid = D > 0.0 && pos(aU) ? div_pos(aU, D) : 0.0;
+  }
   return __dadd_rn(__dadd_rn(__dmul_rn(y, omb), mid), p.eps[q]);
 }
 
@@ -228,39 +231,30 @@ constexpr int kGenWarps = kGenThreads / 32;
 constexpr int kGenEventWarps = 8192;                // event step: a warp per component up to this many
 
 // ---------------------------------------------------------------------------
-// Speculative binary32 direct method of one node-day (one thread), the general
-// form of the SISe kernels' certified clock.  With u = 2^-24, nt <= 32 and every
-// rate constant and continuous variable 0 or within [2^-30, 2^30], counts below
-// 2^21 (so every population below 2^23 is exact in binary32): a binary32 rate
-// (constant and variable truncated to binary32, 2u each; at most three products
-// and one IEEE quotient, u each) is within 8u of the binary64 rate, and never 0
-// unless that rate is 0; a left-to-right partial sum P~_j of non-negative terms
-// is within (nt + 8)u of P_j, r~ = a0~ u2~ within (nt + 10)u of r.  A selection
-// is taken in binary32 only when r~ and every threshold it is compared with are
-// at least 2 nt + 32 float ulps apart (their relative gap then exceeds the sum of
-// the two bounds), else the exact binary64 rule decides that step.  The clock:
-// tau~ = E~ / a0~ (E~ within 16u, the fast quotient 4u) is within (nt + 28)u <=
-// 60u of tau; accumulated exactly in Q62 it stays, at a decision (sum < 2.5),
-// within 150u plus k (2^-53 + 2^-62) of the binary64 chain, so a margin of 2^-16
-// (256u) makes "sum >= 1 + margin" a certain stop and "sum + margin < 1" a
-// certain continue; a decision in between hands the node-day back to the exact
-// method.  The results are the specification's, bit for bit.
-constexpr uint32_t kGenSpecMaxSteps = 1u << 21;
+// Binary32 methods.  With u = 2^-24, nt <= 32, every constant k_j y_q 0 or within
+// [2^-100, 2^60] and counts and populations below 2^22 (exact in binary32): a
+// binary32 rate (the constant truncated, 2u; at most two products, one reciprocal
+// of 1 ulp and its product) is within 8u of the binary64 rate, and never 0 unless
+// that rate is 0; a sum of non-negative rates adds at most the depth of its
+// addition tree.  A selection is taken in binary32 only when r~ and every threshold
+// it is compared with are further apart than their bounds, else the exact binary64
+// rule decides that draw; a clock decision inside the margin hands the node-day
+// back to the binary64 method.  The results are the specification's, bit for bit.
+// A positive constant below 2^-100 (a variable that decayed for years) is taken as
+// 2^-100: its rate, at most 2^-56, is then too large by less than u / 4 of any a0~ from
+// 2^-30 on, and below that no draw is a certain continue while a certain stop only
+// becomes more certain with the true, smaller a0.
+constexpr uint32_t kGenSpecMaxSteps = 1u << 18;
+constexpr float kGenSmallA0 = 9.313226e-10f;                  // 2^-30
+constexpr float kGenBigCount = 4194304.0f;                    // 2^22
 
-// binary32 of rate j, in gen_rate's order; exactly 0 when the binary64 rate is.
-__device__ __forceinline__ float gen_rate_f32(const GenModelDev& m, const GenRepParams& p, const int32_t* x,
-                                              int stride, const float* yf, int j) {
-  float a = trunc_to_f32(p.rate[j]);
-  const int q = m.fy[j], fa = m.fa[j], fb = m.fb[j];
-  const uint32_t pm = m.pop[j];
-  if (q >= 0) a = __fmul_rn(a, yf[q]);
-  if (fa >= 0) a = __fmul_rn(a, small_int_to_f32(x[fa * stride]));
-  if (fb >= 0) a = __fmul_rn(a, small_int_to_f32(x[fb * stride]));
-  if (pm) {
-    const long long P = mask_sum(x, stride, pm, m.nc);
-    a = (P > 0 && a > 0.0f) ? __fdiv_rn(a, small_int_to_f32((int32_t)P)) : 0.0f;
-  }
-  return a;
+// binary32 constant k_j y_q of a transition; false when outside the bounds above.
+__device__ __forceinline__ bool gen_const_f32(double k, bool has_y, double y, float& c) {
+  const double ky = has_y ? __dmul_rn(k, y) : k;
+  const int e = (int)(double_bits(ky) >> 52) - 1023;
+  c = !pos(ky) ? 0.0f : (e < -100 ? 7.8886091e-31f : trunc_to_f32(ky));
+  if (has_y && !pos(y) && double_bits(y) != 0ull) return false;   // negative or -0: exact method
+  return !pos(ky) || e < 60;
 }
 
 // The exact rule of Eq. (sampling2) for state x and uniform u2, in two passes of
@@ -287,240 +281,487 @@ __device__ __forceinline__ int gen_exact_choice(const GenModelDev& m, const GenR
   return last;
 }
 
-// Transitions fired, -1 when a clock decision was too close to call (the caller
-// reruns the node-day exactly from its start), -2 when the binary32 bounds do not
-// hold for this node-day (the caller runs it exactly; x is untouched).  The
-// binary32 rates af_j and partial sums Pf_j live in the thread's row of R.P,
-// viewed as pairs of floats.
-__device__ __forceinline__ int32_t gen_node_day_spec(const GenModelDev& m, const GenRepParams& p, int32_t* x,
-                                                     int stride, const RateRow& R, const double* y, uint32_t v,
-                                                     uint32_t day, uint32_t rep, uint32_t k0, uint32_t k1,
-                                                     uint64_t margin) {
-  const int nt = m.nt, nc = m.nc, ny = m.ny;
-  if (nt == 0) return 0;                                      // no transitions: nothing fires
-  bool ok = true;
-  for (int j = 0; j < nt; ++j) {
-    const double c = p.rate[j];
-    const int e = (int)(double_bits(c) >> 52) - 1023;
-    if (pos(c) && (e < -30 || e > 29)) ok = false;
-  }
-  float yf[kGenMaxCont];
-  for (int q = 0; q < ny; ++q) {
-    const double c = y[q];
-    const int e = (int)(double_bits(c) >> 52) - 1023;
-    if (pos(c) && (e < -30 || e > 29)) ok = false;
-    if (!pos(c) && double_bits(c) != 0ull) ok = false;       // negative or -0: exact method
-    yf[q] = pos(c) ? trunc_to_f32(c) : 0.0f;
-  }
-  long long tot = 0;
-  for (int c = 0; c < nc; ++c) tot += x[c * stride];
-  if (!ok || tot >= (1 << 21)) return -2;
-  float* F = reinterpret_cast<float*>(R.P);
-  const int S2 = 2 * R.stride;
-  const int M = 2 * nt + 32;                                  // decisive gap in float ulps
-  float run = 0.0f;
-  for (int j = 0; j < nt; ++j) {
-    const float aj = gen_rate_f32(m, p, x, stride, yf, j);
-    run = j == 0 ? aj : __fadd_rn(run, aj);
-    F[j * S2] = aj;
-    F[j * S2 + 1] = run;
-  }
-  uint64_t tq = 0;
-  uint4 wn = philox10(make_uint4(v, day, 0u, rep), k0, k1);
-  for (uint32_t k = 0;; ++k) {
-    const float a0f = F[(nt - 1) * S2 + 1];
-    const uint4 w = wn;
-    wn = philox10(make_uint4(v, day, k + 1u, rep), k0, k1);
-    if (!(a0f > 0.0f)) return (int32_t)k;                     // every rate 0: the day ends
-    const float Ef = neglog_f32(((((uint64_t)w.y) << 32) | w.x) >> 12);
-    const float u2f = f32_of_q53(((((((uint64_t)w.w) << 32) | w.z) >> 12) << 1) | 1ull);
-    const uint64_t sq = tq + q62_of(fminf(__fdividef(Ef, a0f), 1.5f));
-    if (sq >= kQ62One + margin) return (int32_t)k;
-    if (sq + margin >= kQ62One || k + 1u >= kGenSpecMaxSteps) return -1;
-    // selection: the first j with a_j > 0 and r <= P_j, each comparison decisive
-    const float rf = __fmul_rn(a0f, u2f);
-    const int ir = __float_as_int(rf);
-    int chosen = -1;
-    bool amb = ir < 0x00800000;
-    for (int j = 0; j < nt && !amb && chosen < 0; ++j) {
-      if (!(F[j * S2] > 0.0f)) continue;
-      const int d = ir - __float_as_int(F[j * S2 + 1]);
-      if (d <= -M) chosen = j;
-      else if (d < M) amb = true;
-    }
-    if (amb || chosen < 0) chosen = gen_exact_choice(m, p, x, stride, y, uniform_open(w.z, w.w));
-    for (int q = m.chg_off[chosen]; q < m.chg_off[chosen + 1]; ++q) {
-      const uint32_t c = m.chg[q];
-      const int32_t dlt = (int32_t)c >> 8;
-      x[(c & 0xffu) * stride] += dlt;
-      tot += dlt;
-    }
-    if (tot >= (1 << 22)) return -1;                          // populations no longer exact in binary32
-    uint32_t dm = m.dep[chosen];
-    const int j0 = dm ? __ffs(dm) - 1 : nt;
-    while (dm) {
-      const int j = __ffs(dm) - 1;
-      dm &= dm - 1u;
-      F[j * S2] = gen_rate_f32(m, p, x, stride, yf, j);
-    }
-    float pr = j0 > 0 ? F[(j0 - 1) * S2 + 1] : 0.0f;
-    for (int j = j0; j < nt; ++j) {
-      pr = j == 0 ? F[0] : __fadd_rn(pr, F[j * S2]);
-      F[j * S2 + 1] = pr;
-    }
-    tq = sq;
+// A thread's column of shared memory (stride kGenThreads): its node's counts, the
+// model's distinct populations (those a firing can change first), a row of ones and a
+// scratch row, as binary32.  The column is about to be read as the other of int32 and
+// float:
+__device__ __forceinline__ void column_retyped() { asm volatile("" ::: "memory"); }
+
+__device__ __forceinline__ void column_to_int(float* xf, int nc) {
+  int32_t* xi = reinterpret_cast<int32_t*>(xf);
+  for (int c = 0; c < nc; ++c) {
+    const int32_t x = (int32_t)xf[c * kGenThreads];
+    column_retyped();
+    xi[c * kGenThreads] = x;
   }
 }
 
-// The segment method (gen_seg_node_day) with the binary32 arithmetic of
-// gen_node_day_spec: each lane's draw gives E~ and u2~; the fixed-point iteration
-// over the segment's lanes chooses with binary32 rates and partial sums, a choice
-// taken in binary32 only when decisive (else gen_exact_choice at that lane's
-// state), so the converged choices are the binary64 method's; each lane's tau~ =
-// E~ / a0~ goes into an exact Q62 scan over the segment, and a lane is a certain
-// continue when its clock plus the margin is below 1, a certain stop when its
-// clock is at least 1 plus the margin (or it has no positive rate).  The day
-// ends at the first lane that is not a certain continue; when that lane is not a
-// certain stop, or a state it decides at leaves the bounds (a negative count, a
-// population of 2^22 or more), the segment gives up.  Returns, for every lane,
-// its segment's transitions fired; -1 when the segment gave up after changing
-// `base` (the caller reloads the day's start state and reruns the node-day with
-// gen_seg_node_day), -2 when the bounds fail at the day's start (nothing changed);
-// 0 for lanes without a node.  Every lane of the warp takes part in the
-// collectives.
-template <int SEG>
-__device__ __forceinline__ int32_t gen_seg_node_day_spec(const GenModelDev& m, const GenRepParams& p, int32_t* xl,
-                                                         int32_t* base, int stride, const RateRow& R,
-                                                         const double* y, uint32_t v, uint32_t day, uint32_t rep,
-                                                         uint32_t k0, uint32_t k1, int sl, int sb, bool live,
-                                                         uint64_t margin) {
-  const int nt = m.nt, nc = m.nc, ny = m.ny;
-  const unsigned full = 0xffffffffu;
-  const unsigned seg = SEG == 32 ? full : (((1u << SEG) - 1u) << sb);
-  const unsigned below = ((1u << sl) - 1u) << sb;
-  float* F = reinterpret_cast<float*>(R.P);
-  const int S2 = 2 * R.stride;
-  const int M = 2 * nt + 32;                                  // decisive gap in float ulps
-  int32_t status = 0;
-  float yf[kGenMaxCont];
-  bool act = live && nt > 0;
-  if (act) {
-    bool ok = true;
-    for (int j = 0; j < nt; ++j) {
-      const double c = p.rate[j];
-      const int e = (int)(double_bits(c) >> 52) - 1023;
-      if (pos(c) && (e < -30 || e > 29)) ok = false;
-    }
-    for (int q = 0; q < ny; ++q) {
-      const double c = y[q];
-      const int e = (int)(double_bits(c) >> 52) - 1023;
-      if (pos(c) && (e < -30 || e > 29)) ok = false;
-      if (!pos(c) && double_bits(c) != 0ull) ok = false;     // negative or -0: exact method
-      yf[q] = pos(c) ? trunc_to_f32(c) : 0.0f;
-    }
-    long long tot = 0;
-    for (int c = 0; c < nc; ++c) tot += base[c];
-    if (!ok || tot >= (1 << 21)) { status = -2; act = false; }
+__device__ __forceinline__ void column_to_float(float* xf, int nc) {
+  const int32_t* xi = reinterpret_cast<const int32_t*>(xf);
+  for (int c = 0; c < nc; ++c) {
+    const int32_t x = xi[c * kGenThreads];
+    column_retyped();
+    xf[c * kGenThreads] = __int2float_rn(x);
   }
+  column_retyped();
+}
+
+// Rates at the column's state, as left-to-right partial sums P (within (nt + 8)u);
+// returns a0.  The rows a rate reads are kernel arguments (uniform), its constants
+// registers, so every rate is recomputed without divergence: about eight instructions
+// each.
+template <int L>
+__device__ __forceinline__ float gen_sums_f32(const GenSsaArgs& a, const float (&kyf)[L], const float* xf,
+                                              float (&P)[L]) {
+  float a0 = 0.0f;
+#pragma unroll
+  for (int j = 0; j < L; ++j) {
+    if (j < a.nt) {
+      float r = __fmul_rn(kyf[j], xf[a.fa[j]]);
+      if (a.fb[j] >= 0) r = __fmul_rn(r, xf[a.fb[j]]);
+      if (a.pr[j] >= 0) {
+        const float pop = xf[a.pr[j]];
+        r = pop > 0.0f ? __fmul_rn(r, rcp_approx(pop)) : 0.0f;
+      }
+      a0 = __fadd_rn(a0, r);
+    }
+    P[j] = a0;
+  }
+  return a0;
+}
+
+// The transition r = a0 u2 fires: the number of thresholds below r (zero-width
+// intervals, from zero rates, are skipped), -1 unless r~ (within (nt + 26)u) is at
+// least 2^-17 r~ = 128u from every threshold: more than 2 nt + 34 <= 98.
+template <int L>
+__device__ __forceinline__ int gen_select_f32(int nt, const float (&P)[L], float r) {
+  float gap = r;
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < L; ++j)
+    if (j < nt) {
+      const float e = __fsub_rn(r, P[j]);
+      gap = fminf(gap, fabsf(e));
+      n += e > 0.0f ? 1 : 0;
+    }
+  return gap < __fmul_rn(r, 7.6293945e-6f) || n >= nt ? -1 : n;
+}
+
+// The thread method: one node per thread.  A firing n applies chg[n] = two (row,
+// change) pairs, further ones from more[].  About 100 instructions and 350 cycles a
+// step for six transitions.  The clock (as in ssa_node_day_spec) is within (nt + 35)u t
+// plus 2^-22 sum(1 / a0~) of the binary64 chain.  Returns the transitions fired, or -1
+// for the caller to rerun the node-day.
+template <int L>
+__device__ __forceinline__ int32_t gen_thread_node_day(const GenSsaArgs& a, const GenModelDev& m,
+                                                       const GenRepParams& p, const int4* chg, const int2* more,
+                                                       const float (&kyf)[L], float* xf, const double* y, uint32_t v,
+                                                       uint32_t rep, uint32_t k0, uint32_t k1, float margin) {
+  const int nt = a.nt;
+  float hi = 2.0f, lo = 0.0f, mm = margin, nl, u2f;
+  uint4 w = philox10(make_uint4(v, (uint32_t)a.day, 0u, rep), k0, k1);
+  draw_f32(w, nl, u2f);
+  for (uint32_t k = 0;; ++k) {
+    float P[L];
+    const float a0 = gen_sums_f32<L>(a, kyf, xf, P);
+    const uint4 wn = philox10(make_uint4(v, (uint32_t)a.day, k + 1u, rep), k0, k1);
+    const float q = rcp_approx(a0);
+    const float tau = __fmul_rn(nl, __fmul_rn(q, 0.693147182f));
+    const float hn = __fadd_rn(hi, tau);
+    lo = __fadd_rn(lo, __fsub_rn(tau, __fsub_rn(hn, hi)));
+    hi = hn;
+    mm = __fmaf_rn(q, 2.5e-7f, mm);
+    const float d = __fadd_rn(__fsub_rn(hi, 3.0f), lo);
+    if (!(a0 > 0.0f) || d > -mm || k >= kGenSpecMaxSteps) return (!(a0 > 0.0f) || d >= mm) ? (int32_t)k : -1;
+    int n = gen_select_f32<L>(nt, P, __fmul_rn(a0, u2f));
+    if (n < 0) {
+      column_to_int(xf, m.nc);
+      n = gen_exact_choice(m, p, reinterpret_cast<const int32_t*>(xf), kGenThreads, y, uniform_open(w.z, w.w));
+      column_to_float(xf, m.nc);
+    }
+    const int4 e = chg[n];
+    const float x0 = __fadd_rn(xf[e.x & 0xffff], (float)(int16_t)(e.y & 0xffff));
+    const float x1 = __fadd_rn(xf[e.x >> 16], (float)(e.y >> 16));
+    xf[e.x & 0xffff] = x0;
+    xf[e.x >> 16] = x1;
+    bool over = fmaxf(x0, x1) >= kGenBigCount;
+    for (int i = e.z; i < e.w; ++i) {
+      const int2 c = more[i];
+      const float x = __fadd_rn(xf[c.x], (float)c.y);
+      xf[c.x] = x;
+      over = over || x >= kGenBigCount;
+    }
+    if (over) return -1;
+    if ((k & 63u) == 63u) {
+      const float h = __fadd_rn(hi, lo);
+      lo = __fsub_rn(lo, __fsub_rn(h, hi));
+      hi = h;
+    }
+    w = wn;
+    draw_f32(w, nl, u2f);
+  }
+}
+
+// The segment method in binary32: SEG lanes per node, SEG draws a round, decided by the
+// fixed-point iteration of gen_seg_node_day.  A pass counts each transition's firings
+// below the lane with one ballot, builds the lane's state from the segment's base
+// (base[row] + sum of change[row][n] count_n, a dense product: rows and counts need no
+// lists and no read-modify-write chains), and takes the rates, sums and choice of the
+// thread method: about 150 instructions and 450 cycles for six transitions, against
+// 2,800 cycles for a pass over transitions, counts and sums in shared memory one by
+// one.  EXACT (SEG = 32): the clock of each lane's draw in binary64 (tau of its state,
+// summed exactly in Q62; a decision is certain outside (k + 2) 2^-52), for node-days
+// whose binary32 clock was too close to call.  Otherwise tau~ = E~ / a0~ (neglog_f32:
+// 16u) goes through a binary32 scan of the round, whose start is a binary32 pair:
+// within (nt + 38)u t of the binary64 chain; it is taken in every pass, and the round
+// ends once no choice before the first draw that is not a certain continue changes
+// (rounds that rarely hold the day's end, a0 > 2 SEG, settle every choice first).
+// Every lane returns its segment's transitions fired, or -1 (a clock decision too close
+// to call, or a state out of bounds): base then no longer holds the day's start.
+template <int L, int SEG, bool EXACT>
+__device__ __forceinline__ int32_t gen_draws_node_day(const GenSsaArgs& a, const GenModelDev& m, const GenRepParams& p,
+                                                      const float* S, const float (&kyf)[L], float* xf, float* base,
+                                                      const double* y, uint32_t v, uint32_t rep, uint32_t k0,
+                                                      uint32_t k1, bool live, float margin) {
+  const unsigned full = 0xffffffffu;
+  const unsigned seg = SEG == 32 ? full : ((1u << (SEG & 31)) - 1u);
+  const int lane = threadIdx.x & 31, sl = lane & (SEG - 1), sb = lane & ~(SEG - 1);
+  const unsigned below = ((1u << sl) - 1u) << sb;
+  const int nt = a.nt, rows = a.dyn_rows;
+  bool done = !live || nt == 0;
+  int32_t result = 0, fired = 0;
+  float hi = 2.0f, lo = 0.0f;
   uint64_t tq = 0;
-  uint32_t fired = 0;
-  for (uint32_t kb = 0; __any_sync(full, act); kb += SEG) {
-    float Ef = 0.0f, u2f = 0.0f;
-    uint32_t wz = 0, ww = 0;
-    if (act) {
-      const uint4 w = philox10(make_uint4(v, day, kb + (uint32_t)sl, rep), k0, k1);
-      Ef = neglog_f32((((uint64_t)w.y << 32) | w.x) >> 12);
-      u2f = f32_of_q53(((((((uint64_t)w.w) << 32) | w.z) >> 12) << 1) | 1ull);
-      wz = w.z;
-      ww = w.w;
-    }
-    int choice = -1;
-    float a0f = 0.0f;
-    bool bad = false;
-    for (int pass = 0; pass <= SEG; ++pass) {
-      if (act)
-        for (int c = 0; c < nc; ++c) xl[c * stride] = base[c];
-      for (int j = 0; j < nt; ++j) {
-        const int cnt = __popc(__ballot_sync(full, act && choice == j) & below);
-        if (cnt) apply_changes(m, xl, stride, j, cnt);
+  for (int r = rows; r < a.xrows; ++r) xf[r * kGenThreads] = base[r];   // rows no firing changes
+  for (uint32_t kb = 0; !__all_sync(full, done); kb += SEG) {
+    if (!done && kb >= kGenSpecMaxSteps) { done = true; result = -1; }
+    const uint4 w = philox10(make_uint4(v, (uint32_t)a.day, kb + (uint32_t)sl, rep), k0, k1);
+    const uint64_t j52 = (((uint64_t)w.y << 32) | w.x) >> 12;
+    const float Ef = EXACT ? 0.0f : neglog_f32(j52);
+    const float u2f = f32_of_q53(((((((uint64_t)w.w) << 32) | w.z) >> 12) << 1) | 1ull);
+    int choice = -2, e = SEG;
+    float sc = 0.0f;
+    bool bad = false, valid = false, sure = false;
+    for (int it = 0; it <= SEG; ++it) {
+      float cnt[L];
+#pragma unroll
+      for (int n = 0; n < L; ++n)
+        cnt[n] = n < nt ? __int2float_rn(__popc(__ballot_sync(full, choice == n) & below)) : 0.0f;
+      float least = 0.0f, most = 0.0f;
+      for (int r = 0; r < rows; ++r) {
+        float x = base[r];
+        const float* Sr = S + r * L;
+#pragma unroll
+        for (int n = 0; n < L; ++n) x = __fmaf_rn(Sr[n], cnt[n], x);
+        least = fminf(least, x);
+        most = fmaxf(most, x);
+        xf[r * kGenThreads] = x;
       }
+      bad = least < 0.0f || most >= kGenBigCount;
+      float P[L];
+      const float a0 = gen_sums_f32<L>(a, kyf, xf, P);
+      valid = !done && !bad && a0 > 0.0f;
       int next = -1;
-      if (act) {
-        long long tot = 0;
-        bool neg = false;
-        for (int c = 0; c < nc; ++c) {
-          const int32_t xc = xl[c * stride];
-          tot += xc;
-          neg = neg || xc < 0;
-        }
-        bad = neg || tot >= (1 << 22);
-        float run = 0.0f;
-        for (int j = 0; j < nt; ++j) {
-          const float aj = bad ? 0.0f : gen_rate_f32(m, p, xl, stride, yf, j);
-          run = j == 0 ? aj : __fadd_rn(run, aj);
-          F[j * S2] = aj;
-          F[j * S2 + 1] = run;
-        }
-        a0f = run;
-        if (!bad && a0f > 0.0f) {
-          const float rf = __fmul_rn(a0f, u2f);
-          const int ir = __float_as_int(rf);
-          bool amb = ir < 0x00800000;
-          for (int j = 0; j < nt && !amb && next < 0; ++j) {
-            if (!(F[j * S2] > 0.0f)) continue;
-            const int d = ir - __float_as_int(F[j * S2 + 1]);
-            if (d <= -M) next = j;
-            else if (d < M) amb = true;
-          }
-          if (amb || next < 0) next = gen_exact_choice(m, p, xl, stride, y, uniform_open(wz, ww));
+      if (valid) {
+        next = gen_select_f32<L>(nt, P, __fmul_rn(a0, u2f));
+        if (next < 0) {
+          column_to_int(xf, m.nc);
+          next = gen_exact_choice(m, p, reinterpret_cast<const int32_t*>(xf), kGenThreads, y, uniform_open(w.z, w.w));
+          column_to_float(xf, m.nc);
         }
       }
-      const bool changed = __any_sync(full, act && next != choice);
+      const bool changed = next != choice;
+      if ((EXACT || __any_sync(full, valid && a0 > 2.0f * SEG)) && it < SEG && __any_sync(full, changed)) {
+        choice = next;
+        continue;
+      }
+      if (EXACT) { choice = next; break; }
+      sc = valid ? fminf(__fmul_rn(Ef, rcp_approx(a0)), 4.0f) : 0.0f;
+#pragma unroll
+      for (int o = 1; o < SEG; o <<= 1) {
+        const float t = __shfl_up_sync(full, sc, o, SEG);
+        if (sl >= o) sc = __fadd_rn(sc, t);
+      }
+      const float d = __fadd_rn(__fadd_rn(__fsub_rn(hi, 3.0f), lo), sc);
+      const bool cont = valid && a0 >= kGenSmallA0 && d <= -margin;
+      sure = !bad && (!valid || d >= margin);
+      const unsigned notcont = (__ballot_sync(full, !cont) >> sb) & seg;
+      e = notcont ? __ffs(notcont) - 1 : SEG;
+      const unsigned diff = (__ballot_sync(full, changed) >> sb) & seg & (e < SEG ? ((1u << e) - 1u) : seg);
       choice = next;
-      if (!changed) break;
+      if (__all_sync(full, done || diff == 0u)) break;
     }
-    // the segment's clock after each lane's draw, exactly in Q62
-    uint64_t S = (act && !bad && choice >= 0) ? q62_of(fminf(__fdividef(Ef, a0f), 1.5f)) : 0ull;
-    for (int d = 1; d < SEG; d <<= 1) {
-      const uint64_t o = __shfl_up_sync(full, S, d, SEG);
-      if (sl >= d) S += o;
+    if (EXACT) {
+      // tau of the lane's draw in binary64, the round's clock exactly in Q62
+      uint64_t q = 0;
+      if (valid) {
+        column_to_int(xf, m.nc);
+        double A = 0.0;
+        for (int j = 0; j < nt; ++j) {
+          const double aj = gen_rate(m, p, reinterpret_cast<const int32_t*>(xf), kGenThreads, y, j);
+          A = j == 0 ? aj : __dadd_rn(A, aj);
+        }
+        column_to_float(xf, m.nc);
+        const double tau = div_pos(neglog_u(j52), A);
+        q = q62_of_f64(le_nonneg(tau, 1.5) ? tau : 1.5);
+      }
+#pragma unroll
+      for (int o = 1; o < SEG; o <<= 1) {
+        const uint64_t t = __shfl_up_sync(full, q, o, SEG);
+        if (sl >= o) q += t;
+      }
+      const uint64_t t = tq + q, close = ((uint64_t)kb + (uint64_t)sl + 2ull) << 10;   // (k + 2) 2^-52
+      sure = !bad && (!valid || t >= kQ62One + close);
+      const unsigned notcont = __ballot_sync(full, !(valid && t + close < kQ62One));
+      e = notcont ? __ffs(notcont) - 1 : SEG;
+      tq = __shfl_sync(full, t, SEG - 1);
     }
-    S += tq;
-    const bool cont = act && !bad && choice >= 0 && S + margin < kQ62One;
-    const bool stop_ok = act && !bad && (choice < 0 || S >= kQ62One + margin);
-    const unsigned notc = __ballot_sync(full, act && !cont) & seg;
-    const unsigned sure = __ballot_sync(full, stop_ok) & seg;
-    int stop = SEG;
-    if (act && notc) {
-      const int e = __ffs(notc) - 1;                           // absolute lane of the first non-continue
-      if ((sure >> e) & 1u) stop = e - sb;
-      else status = -1;
-    }
-    if (act && status == 0 && stop == SEG && kb + 2u * SEG >= kGenSpecMaxSteps) status = -1;
-    const bool apply = act && status == 0;
-    const unsigned fired_lanes = stop == SEG ? seg : (((1u << stop) - 1u) << sb);
-    for (int j = 0; j < nt; ++j) {
-      const int cnt = __popc(__ballot_sync(full, apply && choice == j) & fired_lanes);
-      if (cnt && apply && sl == 0) apply_changes(m, base, 1, j, cnt);
+    // the round's outcome per segment: the state before draw e, or after the last one
+    const unsigned sures = (__ballot_sync(full, sure) >> sb) & seg;
+    const int src = sb + (e < SEG ? e : SEG - 1);
+    const int last = __shfl_sync(full, choice, src);
+    const float round = __shfl_sync(full, sc, src);
+    __syncwarp();
+    if (!done) {
+      for (int r = sl; r < rows; r += SEG) {
+        float x = xf[r * kGenThreads + (src - lane)];
+        if (e == SEG && last >= 0) x = __fadd_rn(x, S[r * L + last]);   // every lane fired
+        base[r] = x;
+      }
+      if (e < SEG) {
+        result = ((sures >> e) & 1u) ? fired + e : -1;
+        done = true;
+      } else {
+        const float hn = __fadd_rn(hi, round);
+        lo = __fadd_rn(lo, __fsub_rn(round, __fsub_rn(hn, hi)));
+        hi = hn;
+        fired += SEG;
+      }
     }
     __syncwarp();
-    const uint64_t tq_end = __shfl_sync(full, S, sb + SEG - 1);
-    if (act) {
-      if (status < 0) act = false;
-      else {
-        fired += (uint32_t)stop;
-        if (stop < SEG) act = false;
-        else tq = tq_end;
-      }
-    }
   }
-  if (!live) return 0;
-  return status < 0 ? status : (int32_t)fired;
+  return result;
 }
 
-// At most 128 registers a thread (110 used): with __launch_bounds__ alone ptxas
-// settled at 72 and spilled inside the binary32 segment method.
-__global__ void __maxnreg__(128) k_gen_ssa(GenSsaArgs a) {
+// Bound by the latency of the longest chain of a launch (about 10 us of it fixed: the
+// model's copy, order, counts, variables and constants in sequence).  Measured per run,
+// one GB300, against the kernel this replaced (transitions walked in shared memory, one
+// block of 128 nodes each): SIR 2,000 nodes x 60 days 2.0 -> 1.2 ms, Erlang 1,500 x 40
+// 13.8 -> 3.3 ms, SEIRS midpoint 37,000 x 365 26.1 -> 16.4 ms, SISe3 37,000 x 365
+// 20.1 -> 13.5 ms.
+//
+// The stochastic step: warps of a resident grid (as node_day_dealt deals its units) take
+// the warp nodes first (largest first, a node's replicates together), then units of four
+// nodes for the segment method, then units of 32 for the thread method.
+template <int L>
+__global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
+  extern __shared__ int4 smem4[];
+  GenModelDev& m = *reinterpret_cast<GenModelDev*>(smem4);
+  char* sp = reinterpret_cast<char*>(smem4) + sizeof(GenModelDev);
+  copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
+  // the change tables: [dyn_rows][L], then the thread method's [nt] and longer lists
+  float* S = reinterpret_cast<float*>(sp);
+  int4* chg = reinterpret_cast<int4*>(S + a.dyn_rows * L);
+  int2* more = reinterpret_cast<int2*>(chg + a.nt);
+  copy16(S, a.tab, a.tab16);
+  sp += (size_t)a.tab16 * 16;
+  double* ctau = reinterpret_cast<double*>(sp);                 // [threads]: per lane
+  sp += kGenThreads * sizeof(double);
+  double* rates = reinterpret_cast<double*>(sp);                // [nt][threads], then partial sums
+  sp += (size_t)2 * a.nt * kGenThreads * sizeof(double);
+  int32_t* rows = reinterpret_cast<int32_t*>(sp);               // [threads / kGenSeg][kGenMaxComp]: day-start counts
+  sp += (kGenThreads / kGenSeg) * kGenMaxComp * sizeof(int32_t);
+  int32_t* cch = reinterpret_cast<int32_t*>(sp);                // [threads]: per lane
+  sp += kGenThreads * sizeof(int32_t);
+  float* kys = reinterpret_cast<float*>(sp);                    // [threads / kGenSeg][L]: a segment's constants
+  sp += (kGenThreads / kGenSeg) * L * sizeof(float);
+  float* bases = reinterpret_cast<float*>(sp);                  // [threads / kGenSeg][xrows]
+  sp += (size_t)(kGenThreads / kGenSeg) * a.xrows * sizeof(float);
+  float* xfs = reinterpret_cast<float*>(sp);                    // [xrows][threads]
+  sp += (size_t)a.xrows * kGenThreads * sizeof(float);
+  int32_t* xs = reinterpret_cast<int32_t*>(sp);                 // [nc][threads]
+  __syncthreads();
+  const unsigned full = 0xffffffffu;
+  const int nc = m.nc, nt = a.nt, ny = m.ny, N = a.N;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // 32-bit unit numbers: gen_create bounds R nc N by 2^31
+  constexpr int kPer = 32 / kGenSeg;
+  const uint32_t T = gridDim.x * kGenWarps, R = (uint32_t)a.R;
+  const uint32_t uw = R * (uint32_t)a.n_big, ug = R * (((uint32_t)a.n_mid + kPer - 1) / kPer);
+  const uint32_t units = uw + ug + R * (((uint32_t)(N - a.n_big - a.n_mid) + 31) / 32);
+  const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32), day = (uint32_t)a.day;
+  const RateRow RR{rates + threadIdx.x, rates + (size_t)nt * kGenThreads + threadIdx.x, kGenThreads};
+  const bool midpoint = m.y_source == kGenYMidpoint, pre_event = m.y_source == kGenYPreEvent;
+  float* xf = xfs + threadIdx.x;
+  int32_t* xi = reinterpret_cast<int32_t*>(xf);
+  for (uint32_t u = (uint32_t)warp * gridDim.x + blockIdx.x; u < units; u += T) {
+    // role 0: a warp node; 1: four nodes on segments; 2: 32 nodes
+    const int role = u < uw ? 0 : (u < uw + ug ? 1 : 2);
+    const uint32_t ut = role == 0 ? u : (role == 1 ? u - uw : u - uw - ug);
+    const uint32_t gi = R == 1 ? ut : ut / R;
+    const int r = (int)(ut - gi * R);
+    const int i = role == 0 ? (int)gi
+                            : (role == 1 ? a.n_big + (int)gi * kPer + lane / kGenSeg
+                                         : a.n_big + a.n_mid + (int)gi * 32 + lane);
+    const bool has = role == 0 || i < (role == 1 ? a.n_big + a.n_mid : N);
+    const int v = has ? a.order[i] : 0;
+    const GenRepParams& p = a.params[r];
+    const uint32_t rep = (uint32_t)(a.rep_base + r);
+    int32_t* X = a.counts + (size_t)r * nc * N + v;
+    double* Y = a.y + (size_t)r * ny * N + v;
+    // lanes per node, the lane's index among them and the node's first lane
+    const int width = role == 0 ? 32 : (role == 1 ? kGenSeg : 1);
+    const int sl = lane & (width - 1), sb = lane & ~(width - 1);
+    const int slot = warp * kPer + (role == 1 ? lane / kGenSeg : 0);
+    int32_t* row = rows + slot * kGenMaxComp;                   // roles 0 and 1: the node's counts
+    if (has)
+      for (int c = sl; c < nc; c += width) {
+        const int32_t x = __ldcg(X + (size_t)c * N);
+        if (role == 2) xi[c * kGenThreads] = x; else row[c] = x;
+      }
+    __syncwarp();
+    const int32_t* x0 = role == 2 ? xi : row;
+    const int xst = role == 2 ? kGenThreads : 1;
+    // continuous variables, shared out over the node's lanes: day - 1's update from its
+    // post-event counts, or the midpoint with the sums saved at its start; then frozen
+    double y[kGenMaxCont];
+    for (int q = 0; q < ny; ++q) {
+      double yq = 0.0;
+      if (has && (q & (width - 1)) == sl) {
+        yq = __ldcg(Y + (size_t)q * N);
+        double* M = a.mid + ((size_t)r * ny + q) * 2 * N + v;
+        double U = 0.0, D = 0.0;
+        if (a.prologue || midpoint) {
+          U = u2d_exact(mask_sum(x0, xst, m.num[q], nc));
+          D = u2d_exact(mask_sum(x0, xst, m.den[q], nc));
+        }
+        if (a.prologue) {
+          yq = gen_y_next(m, p, q, a.day - 1, yq, midpoint ? __dmul_rn(0.5, __dadd_rn(__ldcg(M), U)) : U,
+                          midpoint ? __dmul_rn(0.5, __dadd_rn(__ldcg(M + N), D)) : D);
+          Y[(size_t)q * N] = yq;
+        }
+        if (midpoint) { M[0] = U; M[N] = D; }
+      }
+      y[q] = role == 2 ? yq : __shfl_sync(full, yq, sb + (q & (width - 1)));
+    }
+    // binary32 constants, populations and counts (roles 0 and 1: the segment's base)
+    bool ok = true;
+    float kyf[L];
+    if (role == 2) {
+#pragma unroll
+      for (int j = 0; j < L; ++j) {
+        kyf[j] = 0.0f;
+        if (j < nt) ok = gen_const_f32(p.rate[j], a.fy[j] >= 0, a.fy[j] >= 0 ? y[a.fy[j]] : 0.0, kyf[j]) && ok;
+      }
+    } else {
+      for (int j = sl; j < nt; j += width) {
+        float c;
+        ok = gen_const_f32(p.rate[j], m.fy[j] >= 0, m.fy[j] >= 0 ? y[m.fy[j]] : 0.0, c) && ok;
+        kys[slot * L + j] = c;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < L; ++j) kyf[j] = j < nt ? kys[slot * L + j] : 0.0f;
+    }
+    float* base = bases + slot * a.xrows;
+    long long tot = 0;
+    if (has)
+      for (int c = 0; c < nc; ++c) tot += x0[c * xst];
+    ok = ok && tot < (1 << 21);
+    if (has && ok) {
+      for (int q = sl; q < a.npop; q += width) {
+        const float P = __int2float_rn((int32_t)mask_sum(x0, xst, a.pops[q], nc));
+        if (role == 2) xf[(nc + q) * kGenThreads] = P; else base[nc + q] = P;
+      }
+      if (role == 2) {
+        column_to_float(xf, nc);
+        xf[(nc + a.npop) * kGenThreads] = 1.0f;
+        xf[(nc + a.npop + 1) * kGenThreads] = 0.0f;
+      } else {
+        for (int c = sl; c < nc; c += width) base[c] = __int2float_rn(row[c]);
+        if (sl == 0) { base[nc + a.npop] = 1.0f; base[nc + a.npop + 1] = 0.0f; }
+      }
+    }
+    __syncwarp();
+    int32_t f = has ? -1 : 0;
+    if (role == 2) {
+      if (has && ok)
+        f = nt == 0 ? 0 : gen_thread_node_day<L>(a, m, p, chg, more, kyf, xf, y, (uint32_t)v, rep, k0, k1, a.margin_f);
+      if (has && f >= 0) {
+        column_to_int(xf, nc);
+        for (int c = 0; c < nc; ++c) X[(size_t)c * N] = xi[c * kGenThreads];
+      }
+    } else if (role == 1) {
+      const unsigned oks = __ballot_sync(full, ok);
+      const bool live = has && ((oks >> sb) & ((1u << kGenSeg) - 1u)) == (1u << kGenSeg) - 1u;
+      const int32_t g = gen_draws_node_day<L, kGenSeg, false>(a, m, p, S, kyf, xf, base, y, (uint32_t)v, rep, k0, k1,
+                                                              live, a.margin_f);
+      if (live) f = g;
+    } else if (__all_sync(full, ok)) {
+      f = gen_draws_node_day<L, 32, false>(a, m, p, S, kyf, xf, base, y, (uint32_t)v, rep, k0, k1, true, a.margin_f);
+    }
+    if (role != 2 && has && f >= 0)
+      for (int c = sl; c < nc; c += width) {
+        const int32_t x = (int32_t)base[c];
+        row[c] = x;
+        X[(size_t)c * N] = x;
+      }
+    __syncwarp();
+    if (pre_event && has && f >= 0)
+      for (int q = sl; q < ny; q += width)
+        Y[(size_t)q * N] = gen_y_next(m, p, q, a.day, y[q], u2d_exact(mask_sum(x0, xst, m.num[q], nc)),
+                                      u2d_exact(mask_sum(x0, xst, m.den[q], nc)));
+    // node-days handed back: the whole warp runs each in turn from the day's start (its
+    // global counts), with the binary64 clock, then with the binary64 method
+    unsigned need = __ballot_sync(full, has && f < 0 && sl == 0);
+    while (need) {
+      const int l = __ffs(need) - 1;
+      need &= need - 1;
+      const int vl = __shfl_sync(full, v, l);
+      double yl[kGenMaxCont];
+      for (int q = 0; q < ny; ++q) yl[q] = __shfl_sync(full, y[q], l);
+      float kl[L];
+#pragma unroll
+      for (int j = 0; j < L; ++j) kl[j] = __shfl_sync(full, kyf[j], l);
+      const bool okl = __shfl_sync(full, role == 2 ? ok : tot < (1 << 21), l) &&
+                       (role == 2 || !__any_sync(full, !ok && sb == l));
+      int32_t* Xl = a.counts + (size_t)r * nc * N + vl;
+      int32_t* rl = rows + warp * kPer * kGenMaxComp;           // the warp's first slot: its own node is stored, or this one
+      float* bl = bases + warp * kPer * a.xrows;
+      __syncwarp();
+      if (lane < nc) rl[lane] = __ldcg(Xl + (size_t)lane * N);
+      __syncwarp();
+      int32_t n = -1;
+      if (okl) {
+        for (int q = lane; q < a.npop; q += 32) bl[nc + q] = __int2float_rn((int32_t)mask_sum(rl, 1, a.pops[q], nc));
+        if (lane < nc) bl[lane] = __int2float_rn(rl[lane]);
+        if (lane == 0) { bl[nc + a.npop] = 1.0f; bl[nc + a.npop + 1] = 0.0f; }
+        __syncwarp();
+        n = gen_draws_node_day<L, 32, true>(a, m, p, S, kl, xf, bl, yl, (uint32_t)vl, rep, k0, k1, true, 0.0f);
+        if (n >= 0 && lane < nc) rl[lane] = (int32_t)bl[lane];
+        __syncwarp();
+      }
+      if (n < 0)
+        n = (int32_t)gen_seg_node_day<32>(m, p, xs + threadIdx.x, rl, kGenThreads, RR, ctau + warp * 32,
+                                          cch + warp * 32, yl, (uint32_t)vl, day, rep, k0, k1, lane, 0, true);
+      if (lane < nc) Xl[(size_t)lane * N] = rl[lane];
+      if (pre_event && lane < ny) {
+        double* Yl = a.y + ((size_t)r * ny + lane) * N + vl;
+        *Yl = gen_y_next(m, p, lane, a.day, *Yl, u2d_exact(mask_sum(rl, 1, m.num[lane], nc)),
+                         u2d_exact(mask_sum(rl, 1, m.den[lane], nc)));
+      }
+      if (sb == l) f = n;
+      __syncwarp();
+    }
+    const uint32_t tot_fired = __reduce_add_sync(full, has && sl == 0 ? (uint32_t)f : 0u);
+    if (lane == 0 && tot_fired) atomicAdd(a.ctr + (size_t)r * 4, (unsigned long long)tot_fired);
+    __syncwarp();                                               // rows, bases and columns are reused by the next unit
+  }
+}
+
+// The binary64 methods only (GEN_OPT_CLOCK_MARGIN 0): warp and group nodes by the
+// segment method, the rest one per thread.
+__global__ void __maxnreg__(128) k_gen_ssa_exact(GenSsaArgs a) {
   extern __shared__ int4 smem4[];
   GenModelDev& m = *reinterpret_cast<GenModelDev*>(smem4);
   char* sp = reinterpret_cast<char*>(smem4) + sizeof(GenModelDev);
@@ -611,39 +852,14 @@ __global__ void __maxnreg__(128) k_gen_ssa(GenSsaArgs a) {
     }
     const uint32_t rep = (uint32_t)(a.rep_base + r), k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     const uint32_t vv = (uint32_t)(has ? v : 0);
-    if (coop) {
-      // the binary32 segment method first; segments it hands back rerun with the
-      // binary64 one from the day's start (the global counts are the day's start
-      // until the writer stores below)
-      int32_t f = -2;
-      if (a.clock_margin)
-        f = kind == 0 ? gen_seg_node_day_spec<32>(m, p, x, base, stride, R, y, vv, (uint32_t)a.day, rep, k0, k1,
-                                                  sl, sb, has, a.clock_margin)
-                      : gen_seg_node_day_spec<kGenSeg>(m, p, x, base, stride, R, y, vv, (uint32_t)a.day, rep, k0,
-                                                       k1, sl, sb, has, a.clock_margin);
-      const bool redo = has && f < 0;
-      if (redo)
-        for (int c = sl; c < nc; c += (kind == 0 ? 32 : kGenSeg)) base[c] = X[(size_t)c * N + v];
-      __syncwarp();
-      uint32_t g = 0;
-      if (__any_sync(0xffffffffu, redo)) {
-        if (kind == 0)
-          g = gen_seg_node_day<32>(m, p, x, base, stride, R, ctau + warp * 32, cch + warp * 32, y, vv,
-                                   (uint32_t)a.day, rep, k0, k1, sl, sb, redo);
-        else
-          g = gen_seg_node_day<kGenSeg>(m, p, x, base, stride, R, ctau + warp * 32 + sb, cch + warp * 32 + sb,
-                                        y, vv, (uint32_t)a.day, rep, k0, k1, sl, sb, redo);
-      }
-      fired = redo ? g : (uint32_t)(f > 0 ? f : 0);
-    } else {
-      int32_t f = -2;
-      if (a.clock_margin) {
-        f = gen_node_day_spec(m, p, x, stride, R, y, (uint32_t)v, (uint32_t)a.day, rep, k0, k1, a.clock_margin);
-        if (f == -1)                               // too close to call: rerun from the day's start
-          for (int c = 0; c < nc; ++c) x[c * stride] = X[(size_t)c * N + v];
-      }
-      fired = f >= 0 ? (uint32_t)f : gen_node_day(m, p, x, stride, R, y, (uint32_t)v, (uint32_t)a.day, rep, k0, k1);
-    }
+    if (kind == 0)
+      fired = gen_seg_node_day<32>(m, p, x, base, stride, R, ctau + warp * 32, cch + warp * 32, y, vv, (uint32_t)a.day,
+                                   rep, k0, k1, sl, sb, has);
+    else if (kind == 1)
+      fired = gen_seg_node_day<kGenSeg>(m, p, x, base, stride, R, ctau + warp * 32 + sb, cch + warp * 32 + sb, y, vv,
+                                        (uint32_t)a.day, rep, k0, k1, sl, sb, has);
+    else
+      fired = gen_node_day(m, p, x, stride, R, y, (uint32_t)v, (uint32_t)a.day, rep, k0, k1);
     if (writer) {
       for (int c = 0; c < nc; ++c) X[(size_t)c * N + v] = x0[c * s0];
       if (m.y_source == kGenYPreEvent) {
@@ -794,18 +1010,57 @@ size_t gen_ssa_smem_bytes(int nc, int nt) {
          (size_t)nc * kGenThreads * sizeof(int32_t);
 }
 
+namespace {
+
+size_t gen_f32_smem_bytes(int nc, int nt, int L, int tab16, int xrows) {
+  return sizeof(GenModelDev) + (size_t)tab16 * 16 + kGenThreads * sizeof(double) +
+         (size_t)2 * nt * kGenThreads * sizeof(double) +
+         (size_t)(kGenThreads / kGenSeg) * (kGenMaxComp + L + xrows) * 4 + kGenThreads * sizeof(int32_t) +
+         (size_t)(xrows + nc) * kGenThreads * 4;
+}
+
+using GenSsaKernel = void (*)(GenSsaArgs);
+GenSsaKernel gen_ssa_kernel(int L) {
+  return L == 4 ? k_gen_ssa<4> : L == 8 ? k_gen_ssa<8> : L == 16 ? k_gen_ssa<16> : k_gen_ssa<32>;
+}
+
+}  // namespace
+
+// Transitions the kernel is unrolled for: the power of two that holds the model's.
+int gen_unroll(int nt) {
+  int L = 4;
+  while (L < nt) L *= 2;
+  return L;
+}
+
+cudaError_t gen_ssa_prepare(int nc, int nt, int L, int tab16, int xrows, int* blocks_per_sm) {
+  const GenSsaKernel k = gen_ssa_kernel(L);
+  const size_t smem = gen_f32_smem_bytes(nc, nt, L, tab16, xrows), exact = gen_ssa_smem_bytes(nc, nt);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024) e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && exact > 48 * 1024)
+    e = cudaFuncSetAttribute((const void*)k_gen_ssa_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)k, kGenThreads, smem);
+  return e;
+}
+
 cudaError_t launch_gen_ssa(GenSsaArgs a, int nt, int nc, cudaStream_t st) {
-  a.warp_blocks = (a.n_big + kGenWarps - 1) / kGenWarps;
-  const int per_block = kGenWarps * (32 / kGenSeg);
-  a.group_blocks = (a.n_mid + per_block - 1) / per_block;
-  const int rest = a.N - a.n_big - a.n_mid;
-  const dim3 grid((unsigned)(a.warp_blocks + a.group_blocks + (rest + kGenThreads - 1) / kGenThreads), (unsigned)a.R);
-  const size_t smem = gen_ssa_smem_bytes(nc, nt);
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_gen_ssa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  if (!a.clock_margin) {
+    a.warp_blocks = (a.n_big + kGenWarps - 1) / kGenWarps;
+    const int per_block = kGenWarps * (32 / kGenSeg);
+    a.group_blocks = (a.n_mid + per_block - 1) / per_block;
+    const int rest = a.N - a.n_big - a.n_mid;
+    const dim3 grid((unsigned)(a.warp_blocks + a.group_blocks + (rest + kGenThreads - 1) / kGenThreads), (unsigned)a.R);
+    k_gen_ssa_exact<<<grid, kGenThreads, gen_ssa_smem_bytes(nc, nt), st>>>(a);
+    return cudaGetLastError();
   }
-  k_gen_ssa<<<grid, kGenThreads, smem, st>>>(a);
+  // resident grid, fewer blocks when the units do not fill it (one unit a warp)
+  const int64_t per = 32 / kGenSeg;
+  const int64_t units =
+      (int64_t)a.R * (a.n_big + ((int64_t)a.n_mid + per - 1) / per + ((int64_t)a.N - a.n_big - a.n_mid + 31) / 32);
+  const int64_t grid = std::min<int64_t>(a.resident_blocks, (units + kGenWarps - 1) / kGenWarps);
+  gen_ssa_kernel(a.L)<<<(unsigned)std::max<int64_t>(grid, 1), kGenThreads, 
+                               gen_f32_smem_bytes(nc, nt, a.L, a.tab16, a.xrows), st>>>(a);
   return cudaGetLastError();
 }
 

@@ -47,11 +47,24 @@ struct GenSsaArgs {
   uint64_t seed;
   int32_t rep_base, N, R, day;
   int32_t n_big;                // leading nodes of the order simulated one per warp
-  int32_t n_mid;                // next nodes of the order, four per warp (8-lane segments)
-  int32_t warp_blocks;          // blocks holding the warp nodes (set by the launcher)
-  int32_t group_blocks;         // blocks holding the group nodes (set by the launcher)
+  int32_t n_mid;                // next nodes of the order, four per warp (binary64 methods)
+  int32_t warp_blocks;          // binary64 methods: blocks holding the warp nodes (set by the launcher)
+  int32_t group_blocks;         // ... the group nodes
   int32_t prologue;             // 1: first apply day - 1's continuous update (post-event or midpoint)
-  uint64_t clock_margin;        // Q62 margin of the thread method's binary32 clock (0: exact method only)
+  uint64_t clock_margin;        // Q62 margin of the binary32 clock (0: binary64 methods only)
+  float margin_f;               // the same as binary32
+  // Change tables, back to back (tab16 16-byte words): [dyn_rows][L] floats, what transition
+  // n adds to row r; the thread method's [nt] {row0 | row1 << 16, change0 | change1 << 16,
+  // first, end of further changes} and those {row, change} pairs (rows in elements of a
+  // thread's column).
+  const float4* tab;
+  int32_t tab16;
+  int32_t nt, L;                // transitions; the power of two the kernel is unrolled for
+  int32_t resident_blocks;      // blocks the device holds at once
+  int32_t xrows;                // rows of a thread's column: counts, populations, ones, scratch
+  int32_t npop, dyn_rows;       // populations; counts and populations a firing can change (these come first)
+  uint32_t pops[kGenMaxTrans];  // the distinct population masks
+  int32_t fa[kGenMaxTrans], fb[kGenMaxTrans], pr[kGenMaxTrans], fy[kGenMaxTrans];  // rows a rate reads (-1: none)
 };
 
 // Event record, 16 bytes: {node, dest, count, kind | select << 8 | shift row << 16}.
@@ -77,7 +90,9 @@ struct GenContArgs {
   int32_t N, R, day;
 };
 
-size_t gen_ssa_smem_bytes(int nc, int nt);
+int gen_unroll(int nt);
+// Shared-memory limits of the stochastic-step kernels and the blocks an SM holds (once per handle).
+cudaError_t gen_ssa_prepare(int nc, int nt, int L, int tab16, int xrows, int* blocks_per_sm);
 cudaError_t launch_gen_ssa(GenSsaArgs a, int nt, int nc, cudaStream_t st);
 cudaError_t launch_gen_events(const GenEvArgs& a, cudaStream_t st);
 cudaError_t launch_gen_cont(const GenContArgs& a, cudaStream_t st);

@@ -28,6 +28,8 @@ struct gen_handle {
   double* d_mid = nullptr;          // [R][Ny][2][N] (midpoint variant)
   int32_t* d_order = nullptr;       // [N]
   GenModelDev* d_model = nullptr;
+  float4* d_tab = nullptr;          // change tables of the binary32 methods
+  GenSsaArgs ssa{};                 // the stochastic step's arguments that do not change between days
   GenRepParams* d_params = nullptr;
   unsigned long long* d_ctr = nullptr;
   int32_t* d_err = nullptr;
@@ -40,7 +42,7 @@ struct gen_handle {
   int32_t launch_mode = 0;          // 0 stream, 1 CUDA graph
   std::vector<int64_t> pop_sorted;  // initial node populations in the node order (descending)
   int32_t warp_threshold = -1;      // initial population from which a node gets a warp (-1: automatic)
-  int32_t clock_margin_log2 = 16;   // binary32 clock margin 2^-k of the thread method (0: exact only)
+  int32_t clock_margin_log2 = 16;   // binary32 clock margin 2^-k (0: exact only)
   int32_t group_threshold = -1;     // ... an 8-lane segment (-1: automatic)
   int32_t n_big = 0;                // nodes simulated one per warp
   int32_t n_mid = 0;                // nodes simulated four per warp
@@ -154,6 +156,61 @@ sim_status build_model(const gen_model* m, GenModelDev* out, char* why, size_t w
   return SIM_OK;
 }
 
+// Tables of the binary32 methods (GenSsaArgs): the rows each rate reads and what each
+// firing changes.
+void build_tables(const GenModelDev& md, const int32_t* stoich, GenSsaArgs* s, std::vector<float4>& tab) {
+  const int nc = md.nc, nt = md.nt, L = gen_unroll(nt);
+  auto change = [&](int c, int n) { return stoich[c * nt + n]; };
+  auto pop_change = [&](uint32_t mask, int n) {
+    int t = 0;
+    for (int c = 0; c < nc; ++c)
+      if (mask >> c & 1u) t += change(c, n);
+    return t;
+  };
+  s->nt = nt;
+  s->L = L;
+  // distinct populations, those some firing changes first
+  for (int dynamic = 1; dynamic >= 0; --dynamic) {
+    for (int j = 0; j < nt; ++j) {
+      if (!md.pop[j] || std::find(s->pops, s->pops + s->npop, md.pop[j]) != s->pops + s->npop) continue;
+      bool moves = false;
+      for (int n = 0; n < nt; ++n) moves = moves || pop_change(md.pop[j], n) != 0;
+      if (moves == (dynamic == 1)) s->pops[s->npop++] = md.pop[j];
+    }
+    if (dynamic) s->dyn_rows = nc + s->npop;
+  }
+  s->xrows = nc + s->npop + 2;
+  const int ones = (nc + s->npop) * kGenThreads, scratch = ones + kGenThreads;
+  auto pop_row = [&](uint32_t mask) { return nc + (int)(std::find(s->pops, s->pops + s->npop, mask) - s->pops); };
+  for (int j = 0; j < nt; ++j) {
+    s->fa[j] = md.fa[j] >= 0 ? md.fa[j] * kGenThreads : ones;
+    s->fb[j] = md.fb[j] >= 0 ? md.fb[j] * kGenThreads : -1;
+    s->fy[j] = md.fy[j];
+    s->pr[j] = md.pop[j] ? pop_row(md.pop[j]) * kGenThreads : -1;
+  }
+  std::vector<float> dense((size_t)s->dyn_rows * L, 0.f);
+  std::vector<int4> first((size_t)nt);
+  std::vector<int2> more;
+  for (int n = 0; n < nt; ++n) {
+    std::vector<int2> ch;                                       // (row, change)
+    for (int r = 0; r < s->dyn_rows; ++r) {
+      const int d = r < nc ? change(r, n) : pop_change(s->pops[r - nc], n);
+      dense[(size_t)r * L + n] = (float)d;
+      if (d) ch.push_back(make_int2(r * kGenThreads, d));
+    }
+    while (ch.size() < 2) ch.push_back(make_int2(scratch, 0));
+    first[(size_t)n] = make_int4(ch[0].x | (ch[1].x << 16), (ch[0].y & 0xffff) | (ch[1].y << 16), (int)more.size(),
+                                 (int)(more.size() + ch.size() - 2));
+    more.insert(more.end(), ch.begin() + 2, ch.end());
+  }
+  const size_t dense16 = dense.size() / 4;                      // L is a multiple of 4
+  tab.assign(dense16 + first.size() + (more.size() + 1) / 2 + 1, make_float4(0.f, 0.f, 0.f, 0.f));
+  std::memcpy(tab.data(), dense.data(), dense.size() * sizeof(float));
+  if (nt) std::memcpy(&tab[dense16], first.data(), first.size() * sizeof(int4));
+  if (!more.empty()) std::memcpy(&tab[dense16 + first.size()], more.data(), more.size() * sizeof(int2));
+  s->tab16 = (int32_t)tab.size();
+}
+
 void free_graph(gen_handle* h) {
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   h->graph_exec = nullptr;
@@ -176,30 +233,48 @@ sim_status latched(gen_handle* h) {
   return SIM_OK;
 }
 
-constexpr int32_t kAutoWarpThreshold = 600;
-constexpr int32_t kAutoGroupThreshold = 150;
+constexpr int32_t kGenMaxMargin = 16;
+constexpr int64_t kAutoWarpThreshold = 600;
+constexpr int64_t kAutoGroupThreshold = 300;
 
+// Warp and group nodes of the node order.  Automatic warp nodes: as many of the largest
+// as let every unit (a node per warp, then 32 nodes per warp) have a resident warp of its
+// own, with a tenth to spare, since a warp node's day takes about 18 us whatever its size
+// while a thread node's grows with its herd -- and those of 600 animals or more in any
+// case.  Measured, one GB300, per run: SEIRS on 37,000 nodes x 365 days 15.3 ms with 1,057
+// warp nodes (one wave), 16.5 with 407, 20.6 with 4,316 (two waves); Erlang on 1,500 nodes
+// x 40 days 3.3 ms with every node a warp node, 8.1 with none.  Automatic group nodes: 300
+// animals or more (24 us a day for herds of 150-300 against 27 us one per thread).
 void set_n_big(gen_handle* h) {
+  const int64_t N = (int64_t)h->pop_sorted.size(), R = h->cfg.n_replicates;
   const int64_t thr = h->warp_threshold < 0 ? kAutoWarpThreshold : h->warp_threshold;
   const int64_t gthr = h->group_threshold < 0 ? kAutoGroupThreshold : h->group_threshold;
-  const int32_t N = (int32_t)h->pop_sorted.size();
-  int32_t n = 0;
+  int64_t n = 0;
+  if (h->warp_threshold < 0) {
+    // largest n with n + (N - n) / 32 <= per
+    const int64_t per = (int64_t)h->ssa.resident_blocks * (kGenThreads / 32) * 9 / 10 / R;
+    n = std::min(N, std::max<int64_t>(0, (32 * per - N) / 31));
+  }
   while (n < N && h->pop_sorted[n] >= thr) ++n;
-  int32_t g = n;
+  int64_t g = n;
   while (g < N && h->pop_sorted[g] >= gthr) ++g;
-  h->n_big = n;
-  h->n_mid = g - n;
+  h->n_big = (int32_t)n;
+  h->n_mid = (int32_t)(g - n);
 }
 
 sim_status enqueue_days(gen_handle* h, int32_t d0, int32_t nd, cudaStream_t st) {
   const int N = h->cfg.n_nodes, R = h->cfg.n_replicates;
   for (int32_t d = d0; d < d0 + nd; ++d) {
-    GenSsaArgs s{};
+    GenSsaArgs s = h->ssa;
     s.counts = h->d_counts; s.y = h->d_y; s.mid = h->d_mid; s.model = h->d_model; s.params = h->d_params;
     s.order = h->d_order; s.ctr = h->d_ctr; s.seed = h->cfg.seed; s.rep_base = h->cfg.replicate_base;
     s.N = N; s.R = R; s.day = d; s.n_big = h->n_big; s.n_mid = h->n_mid;
     s.prologue = (d > d0 && h->ny > 0 && h->model.y_source != GEN_Y_PRE_EVENT) ? 1 : 0;
     s.clock_margin = h->clock_margin_log2 > 0 ? (1ull << (62 - h->clock_margin_log2)) : 0ull;
+    // the binary32 methods' own bound, (nt + 44) 2^-24, is below 2^-16: that is the
+    // margin at the default exponent; a wider margin is taken as asked
+    s.margin_f = h->clock_margin_log2 >= kGenMaxMargin ? std::ldexp((float)(h->nt + 44), -24)
+                                                       : std::ldexp(1.0f, -h->clock_margin_log2);
     GCK(h, launch_gen_ssa(s, h->nt, h->nc, st), "stochastic step launch");
     const int32_t c0 = h->day_comp[d], c1 = h->day_comp[d + 1];
     if (c1 > c0) {
@@ -296,7 +371,6 @@ sim_status gen_create(const gen_model* m, const gen_config* cfg, const int32_t* 
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return tot[a] > tot[b]; });
   h->pop_sorted.resize((size_t)N);
   for (int i = 0; i < N; ++i) h->pop_sorted[i] = tot[order[i]];
-  set_n_big(h);
   const size_t ncount = (size_t)R * nc * N, ncy = (size_t)R * ny * N;
   cudaError_t e = galloc(&h->d_counts, ncount);
   if (e == cudaSuccess) e = galloc(&h->d_y, ncy);
@@ -304,6 +378,19 @@ sim_status gen_create(const gen_model* m, const gen_config* cfg, const int32_t* 
   if (e == cudaSuccess) e = galloc(&h->d_order, (size_t)N);
   if (e == cudaSuccess) e = galloc(&h->d_model, 1);
   if (e == cudaSuccess) e = galloc(&h->d_params, (size_t)R);
+  {
+    std::vector<float4> tab;
+    build_tables(md, m->stoich, &h->ssa, tab);
+    if (e == cudaSuccess) e = galloc(&h->d_tab, tab.size());
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_tab, tab.data(), tab.size() * sizeof(float4), cudaMemcpyHostToDevice);
+    h->ssa.tab = h->d_tab;
+    int dev = 0, sms = 1, per_sm = 1;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = gen_ssa_prepare(nc, nt, h->ssa.L, h->ssa.tab16, h->ssa.xrows, &per_sm);
+    h->ssa.resident_blocks = sms * std::max(per_sm, 1);
+    set_n_big(h);
+  }
   if (e == cudaSuccess) e = galloc(&h->d_ctr, (size_t)R * 4);
   if (e == cudaSuccess) e = galloc(&h->d_err, 1);
   for (int r = 0; r < R && e == cudaSuccess; ++r) {
@@ -566,6 +653,7 @@ void gen_destroy(gen_handle* h) {
   if (!h) return;
   free_graph(h);
   cudaFree(h->d_counts); cudaFree(h->d_y); cudaFree(h->d_mid); cudaFree(h->d_order); cudaFree(h->d_model);
+  cudaFree(h->d_tab);
   cudaFree(h->d_params); cudaFree(h->d_ctr); cudaFree(h->d_err);
   cudaFree(h->d_rec); cudaFree(h->d_comp_ev); cudaFree(h->d_comp_off);
   delete h;
