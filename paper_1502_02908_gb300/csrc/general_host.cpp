@@ -602,8 +602,7 @@ sim_status gen_set_state(gen_handle* h, const int32_t* counts, const double* y, 
   GCK(h, cudaMemcpyAsync(h->d_counts, counts, nx * 4, k, st), "copy counts");
   if (nyv) GCK(h, cudaMemcpyAsync(h->d_y, y, nyv * 8, k, st), "copy y");
   GCK(h, cudaStreamSynchronize(st), "stream synchronize");
-  free_graph(h);
-  h->day = day;
+  h->day = day;                     // a captured day loop reads the state's buffers: it stays valid
   return SIM_OK;
 }
 
