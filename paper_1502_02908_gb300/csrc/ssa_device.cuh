@@ -485,8 +485,233 @@ __device__ __forceinline__ int32_t ssa_node_day_spec(const DevParams& p, uint64_
   return result;
 }
 
-// Warp-cooperative direct method for one node-day (large herds), all 32 lanes
-// together; phases per block of 32 draws:
+// ---------------------------------------------------------------------------
+// The warp method's binary32 tier: 32 draws a round, decided by the fixed-point
+// iteration over the lanes (ssa_warp_node_day below), with two clocks.
+//
+// In a round's passes, a binary32 clock: tau~ = E~ / a0~ (E~ within u and 2^-38, a0~
+// 6u, the reciprocal 2u, the product u) scanned over the round (5u) and added to the
+// round's start (u): within 20u plus 2^-38 sum(1 / a0~) of the binary64 chain, against
+// a margin of 2^-17 = 128u.  The first draw that is not a certain continue ends the
+// day when it is a certain stop.
+//
+// Between rounds, and where the binary32 clock cannot tell, a fixed-point clock
+// (kTauOne = 1 day): E to 2^-38 from a table of 128 reciprocals and a quartic series in
+// 32-bit integers, a0 as a sum of 64-bit fixed-point rates (relative error below
+// 2^-36 while it is at least herd 2^36 units, else the draw is left undecided), and
+// the quotient from a reciprocal corrected by one residual (2^-41).  After k draws it
+// is within 2^-35 + k 2^-48 + 2^-38 sum(1 / a0) of the binary64 chain (k 2^-53 of which
+// is the chain's own rounding); twice that is the margin, so a node-day of 2,000
+// transitions is handed back to the binary64 tiers about once in 10^6 days, and no
+// earlier round is ever replayed.  (A binary32 clock over every round left 3 % of such
+// node-days undecided; replaying their 63 rounds in binary64 took as long as the step
+// itself: 1,000 nodes of 2,000 animals at unit rates, S.)
+constexpr int kTauBits = 56;
+constexpr int64_t kTauOne = 1ll << kTauBits;
+
+// -log(u) 2^43 for u = (2j+1) 2^-53, within 2^-38 (2^5 units); at least 0.  x = 2j+1 =
+// 2^n m: E = (53-n) ln2 - ln m, ln m = ln(1 + z) + L_i with z = m R_i / 1024 - 1, |z| <
+// 2^-7.8, and ln(1 + z) = z - z^2 (1/2 - z (1/3 - z/4)) + O(z^5 / 5 < 2^-41).
+__device__ __forceinline__ uint64_t neglog_q43(uint64_t j) {
+  const uint64_t x = (j << 1) | 1ull;
+  const int lz = __clzll(x);
+  const uint64_t M = x << lz;
+  const int i = (int)(M >> 56) & 127;
+  const int64_t zq = (int64_t)((M >> 15) * (uint64_t)(uint32_t)__ldg(&kRecip[i])) - (int64_t)(1ull << 58);   // Q58
+  const int32_t z = (int32_t)(zq >> 20);                                     // Q38
+  const int32_t t = 715827883 - (z >> 9);                                    // 1/3 - z/4, Q31
+  const int32_t h = (1 << 30) - (__mulhi(z, t) >> 6);                        // 1/2 - z t, Q31
+  const int32_t w = __mulhi(__mulhi(z, z), h);                               // z^2 h, Q43 (z^2 in Q44)
+  const int64_t lnm = (zq >> 15) - (int64_t)w + (__ldg(&kLogR[i]) >> 19);
+  const int64_t e = (int64_t)(lz - 10) * (int64_t)((EPISIM_LN2_Q62 + (1ull << 18)) >> 19) - lnm;   // 53 - n = lz - 10
+  return (uint64_t)(e > 0 ? e : 0);
+}
+
+// floor(c 2^s) of a non-negative binary64 c < 2^(62-s).
+__device__ __forceinline__ uint64_t rate_fixed(double c, int s) {
+  const uint64_t b = double_bits(c);
+  const int e = (int)(b >> 52);
+  if (e == 0) return 0ull;                          // 0 (spec_constants rules out subnormal constants)
+  const uint64_t m = (b & ((1ull << 52) - 1)) | (1ull << 52);
+  const int sh = s + e - 1023 - 52;
+  return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> (-sh)) : 0ull);
+}
+
+// E / a0 in units of 1 / kTauOne (at most 4 days), E = e43 2^-43, a0 = A 2^-s >= 2^-13.
+__device__ __forceinline__ int64_t tau_fixed(uint64_t e43, uint64_t A, int s) {
+  const int lz = __clzll(A);
+  const uint64_t An = A << lz;                      // a0 = An 2^-63 2^ex
+  const int ex = 63 - lz - s;
+  const float ah = __fmul_rn(__uint2float_rn((uint32_t)(An >> 40)), 1.1920929e-7f);                 // in [1, 2)
+  const float al = __fmul_rn(__uint2float_rn((uint32_t)(An >> 8)), 2.7755576e-17f);                 // 2^-55
+  const uint32_t et = (uint32_t)(e43 >> 17) & ~0xFFu;
+  const float eh = __fmul_rn(__uint2float_rn(et), 1.4901161e-8f);                                   // 2^-26, exact
+  const float el = __fmul_rn(__uint2float_rn((uint32_t)(e43 - ((uint64_t)et << 17))), 1.1368684e-13f);  // 2^-43
+  const float q = rcp_approx(ah);
+  const float res = __fmaf_rn(-q, al, __fmaf_rn(-q, ah, 1.0f));
+  const float p = __fmul_rn(eh, q);
+  const float t = __fadd_rn(__fmaf_rn(eh, q, -p), __fmaf_rn(el, q, __fmul_rn(p, res)));
+  const float sc = __uint_as_float((uint32_t)(127 + kTauBits - ex) << 23);
+  return __float2ll_rn(fminf(__fmul_rn(p, sc), 4.0f * (float)kTauOne)) + __float2ll_rn(__fmul_rn(t, sc));
+}
+
+template <int NA>
+__device__ __forceinline__ int32_t ssa_warp_day_spec(const DevParams& p, uint64_t seed, uint32_t rep, int v, int day,
+                                                     double phi, float margin, NodeState<NA>& s) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t full = 0xffffffffu, below = (1u << lane) - 1u;
+  float cinff[NA], gamf[NA];
+  uint64_t Cq[NA], Gq[NA], least;
+  int sq;
+  {
+    double cinf[NA];
+    int32_t herd = 0;
+    int top = -200;
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+      cinf[j] = __dmul_rn(p.ups[j], phi);
+      herd += s.x[2 * j] + s.x[2 * j + 1];
+      top = max(top, max((int)(double_bits(cinf[j]) >> 52), (int)(double_bits(p.gam[j]) >> 52)) - 1022);   // < 2^top
+    }
+    if (!spec_constants<NA>(p, cinf, s.x, cinff, gamf)) return -1;
+    sq = 62 - max(top, -100) - (32 - __clz(herd));   // the rates' sum stays below 2^62 units
+#pragma unroll
+    for (int j = 0; j < NA; ++j) { Cq[j] = rate_fixed(cinf[j], sq); Gq[j] = rate_fixed(p.gam[j], sq); }
+    least = (uint64_t)herd << 36;
+  }
+  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+  int64_t tq = 0;                                   // the clock at the round's start
+  float rsum = 0.0f;                                // bound of sum(1 / a0~) over the earlier rounds
+  int32_t fired = 0;
+  for (uint32_t kb = 0; kb < kFastMaxSteps; kb += 32) {
+    const uint4 w = philox10(make_uint4((uint32_t)v, (uint32_t)day, kb + (uint32_t)lane, rep), k0, k1);
+    const uint64_t e43 = neglog_q43(((((uint64_t)w.y) << 32) | w.x) >> 12);
+    const float Ef = __fmul_rn(__ull2float_rn(e43), 1.1368684e-13f);
+    const float u2f = f32_of_q53(((((((uint64_t)w.w) << 32) | w.z) >> 12) << 1) | 1ull);
+    const float d0 = __fmul_rn(__ll2float_rn(tq - kTauOne), 1.3877788e-17f);   // 2^-56
+    int ch = -3, e = 32, net[NA];
+    bool settle = false, valid = false, sure = false;
+    float q = 0.0f, a0_last = 0.0f;
+    // passes until every choice that matters is settled; `settle`: every lane's choice,
+    // before the clock is taken (rounds that rarely hold the day's end, a0 > 64, and
+    // rounds whose end the binary32 clock cannot decide)
+    int pass = 0;
+    for (;; ++pass) {
+      if (pass > 80) return -1;                     // cannot happen (33 passes settle a round, twice)
+      float S[NA], I[NA], T[2 * NA - 1], a0 = 0.0f;
+#pragma unroll
+      for (int j = 0; j < NA; ++j) {
+        const int inf = __popc(__ballot_sync(full, ch == 2 * j) & below);
+        const int rec = __popc(__ballot_sync(full, ch == 2 * j + 1) & below);
+        net[j] = rec - inf;
+        S[j] = __fadd_rn(__int_as_float(0x4B400000 + s.x[2 * j] + net[j]), -12582912.0f);
+        I[j] = __fadd_rn(__int_as_float(0x4B400000 + s.x[2 * j + 1] - net[j]), -12582912.0f);
+        const float ai = __fmul_rn(cinff[j], S[j]);
+        const float A = __fmaf_rn(gamf[j], I[j], ai);
+        T[2 * j] = j == 0 ? ai : __fadd_rn(a0, ai);
+        a0 = j == 0 ? A : __fadd_rn(a0, A);
+        if (2 * j + 1 < 2 * NA - 1) T[2 * j + 1 < 2 * NA - 1 ? 2 * j + 1 : 0] = a0;
+      }
+      valid = a0 > 0.0f;
+      a0_last = a0;
+      const float r = __fmul_rn(a0, u2f);
+      float gap = r;
+      int nc = 0;
+#pragma unroll
+      for (int i = 0; i < 2 * NA - 1; ++i) {
+        const float dr = __fsub_rn(r, T[i]);
+        gap = fminf(gap, fabsf(dr));
+        nc += dr > 0.0f ? 1 : 0;
+      }
+      if (!valid) nc = -2;
+      else if (gap < __fmul_rn(r, 3.8146973e-6f)) {
+        double cinf[NA];
+        int32_t xs[2 * NA];
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          cinf[j] = __dmul_rn(p.ups[j], phi);
+          xs[2 * j] = s.x[2 * j] + net[j];
+          xs[2 * j + 1] = s.x[2 * j + 1] - net[j];
+        }
+        nc = exact_choice<NA>(cinf, p, xs, uniform_open(w.z, w.w));
+      }
+      if (pass == 0) settle = __shfl_sync(full, a0, 0) > 64.0f;
+      if (settle) {
+        if (__ballot_sync(full, nc != ch)) { ch = nc; continue; }
+        q = valid ? rcp_approx(a0) : 0.0f;
+        break;
+      }
+      q = valid ? rcp_approx(a0) : 0.0f;
+      float sc = fminf(__fmul_rn(Ef, q), 4.0f);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(full, sc, o);
+        if (lane >= o) sc = __fadd_rn(sc, y);
+      }
+      const float d = __fadd_rn(d0, sc);
+      const unsigned notcont = __ballot_sync(full, !(a0 >= 2.44140625e-4f && d <= -margin));
+      const unsigned sures = __ballot_sync(full, !valid || d >= margin);
+      e = notcont ? __ffs(notcont) - 1 : 32;
+      const unsigned diff = __ballot_sync(full, nc != ch) & (e < 32 ? ((1u << e) - 1u) : full);
+      ch = nc;
+      if (diff) continue;
+      if (e == 32) break;                           // the whole round continues
+      if ((sures >> e) & 1u) {
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          const int n = __shfl_sync(full, net[j], e);
+          s.x[2 * j] += n;
+          s.x[2 * j + 1] -= n;
+        }
+        return fired + e;
+      }
+      settle = true;                                // too close to call: the fixed-point clock
+    }
+    // every choice is settled: the round's fixed-point clock
+    uint64_t A = 0;
+#pragma unroll
+    for (int j = 0; j < NA; ++j)
+      A += Cq[j] * (uint64_t)(uint32_t)(s.x[2 * j] + net[j]) + Gq[j] * (uint64_t)(uint32_t)(s.x[2 * j + 1] - net[j]);
+    const bool exact = a0_last >= 2.44140625e-4f && A >= least;
+    int64_t t = exact ? tau_fixed(e43, A, sq) : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(full, t, o);
+      if (lane >= o) t += y;
+    }
+    t += tq;
+    rsum = __fmaf_rn(32.0f, __uint_as_float(__reduce_max_sync(full, __float_as_uint(q))), rsum);
+    if (!(rsum < 524288.0f)) return -1;             // 2^19: the binary32 clock's 2^-38 sum stays below 2^-18
+    // margin 2^-34 + k 2^-47 + 2^-37 sum(1 / a0~), rounded up
+    const int64_t mt = (1ll << (kTauBits - 34)) + ((int64_t)(kb + 32u) << (kTauBits - 47)) +
+                       (int64_t)__fmul_ru(rsum, 524288.0f) + 1;
+    const unsigned notcont = __ballot_sync(full, !(exact && t <= kTauOne - mt));
+    if (notcont) {
+      e = __ffs(notcont) - 1;
+      sure = !valid || (exact && t >= kTauOne + mt);
+      if (!((__ballot_sync(full, sure) >> e) & 1u)) return -1;
+#pragma unroll
+      for (int j = 0; j < NA; ++j) {
+        const int n = __shfl_sync(full, net[j], e);
+        s.x[2 * j] += n;
+        s.x[2 * j + 1] -= n;
+      }
+      return fired + e;
+    }
+    tq = __shfl_sync(full, t, 31);
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+      const int n = __popc(__ballot_sync(full, ch == 2 * j + 1)) - __popc(__ballot_sync(full, ch == 2 * j));
+      s.x[2 * j] += n;
+      s.x[2 * j + 1] -= n;
+    }
+    fired += 32;
+  }
+  return -1;
+}
+
+// Warp-cooperative direct method for one node-day with a binary64 clock (the tiers
+// behind ssa_warp_day_spec), all 32 lanes together; phases per block of 32 draws:
 //  1. lane l computes draw k0 + l: Philox, E = -log(u1), u2 (independent of the
 //     state, so all 32 in parallel);
 //  2. the embedded jump chain (which transition each draw fires): binary32
@@ -494,19 +719,15 @@ __device__ __forceinline__ int32_t ssa_node_day_spec(const DevParams& p, uint64_
 //     (relative gap >= 2^-18, beyond the <= 2^-20 error of the binary32 rates,
 //     sums and product against the specification's binary64 values); otherwise
 //     that draw is decided with the specification's binary64 arithmetic.  With
-//     CLOCK > 0 all lanes decide at once by the fixed-point iteration below; with
+//     CLOCK = 1 all lanes decide at once by the fixed-point iteration below; with
 //     CLOCK = 0 the lanes walk the chain in draw order;
-//  3-4. the clock.  CLOCK = 2: lane l forms tau~_l from its draw's binary32
-//     propensity sum; an inclusive warp scan of the Q62 values gives the clock
-//     after every draw, and the first draw that is not a certain continue ends
-//     the day (certain stop) or returns -1 (too close to call).  CLOCK = 1: the
-//     same scan of the exact binary64 tau_l (a0 of the lane's state, the exact
-//     -log), whose sum is within (k + 2) 2^-53 of the binary64 chain, so only a
-//     decision within that of the day's end returns -1.  CLOCK = 0: the binary64
-//     clock t + tau_l runs in draw order; the first draw reaching t >= 1 ends the
-//     day in the state before that draw.
-// Returns the transitions fired, or -1 (CLOCK > 0) for the caller to rerun the
-// node-day with a smaller CLOCK from the same state.
+//  3-4. the clock.  CLOCK = 1: an inclusive warp scan in Q62 of the exact binary64
+//     tau_l (a0 of the lane's state, the exact -log), whose sum is within
+//     (k + 2) 2^-53 of the binary64 chain, so only a decision within that of the
+//     day's end returns -1.  CLOCK = 0: the binary64 clock t + tau_l runs in draw
+//     order; the first draw reaching t >= 1 ends the day in the state before it.
+// Returns the transitions fired, or -1 (CLOCK = 1) for the caller to rerun the
+// node-day with CLOCK = 0 from the same state.
 // floor(x 2^62) for a non-negative binary64 x <= 1.5 (exact bits).
 __device__ __forceinline__ uint64_t q62_of_f64(double x) {
   const uint64_t b = double_bits(x);
@@ -516,17 +737,9 @@ __device__ __forceinline__ uint64_t q62_of_f64(double x) {
   return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> (-sh)) : 0ull);
 }
 
-// Rounds of the binary32 clock whose choices a warp logs, so that a day end too
-// close to call resumes with the binary64 clock from that round instead of
-// rerunning the node-day.
-constexpr int kReplayRounds = 128;
-
-// Returns the transitions fired, or -1.  kb0, tq0, fired0: resume at draw kb0
-// (a multiple of 32) with the clock tq0 (Q62) and fired0 transitions behind.
 template <int NA, int CLOCK>
 __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_t seed, uint32_t rep, int v, int day,
-                                                     double phi, uint64_t margin, NodeState<NA>& s,
-                                                     uint32_t kb0 = 0, uint64_t tq0 = 0, int32_t fired0 = 0) {
+                                                     double phi, NodeState<NA>& s) {
   constexpr int NC = 2 * NA;
   const int lane = threadIdx.x & 31;
   const uint32_t full = 0xffffffffu;
@@ -534,145 +747,27 @@ __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_
   float cinff[NA], gamf[NA];
 #pragma unroll
   for (int j = 0; j < NA; ++j) cinf[j] = __dmul_rn(p.ups[j], phi);
-  constexpr bool SPEC = CLOCK == 2;
   const bool spec_ok = spec_constants<NA>(p, cinf, s.x, cinff, gamf);
-  if (SPEC && !spec_ok) return -1;
   bool cpos[NA], gpos[NA];
 #pragma unroll
   for (int j = 0; j < NA; ++j) { cpos[j] = pos(cinf[j]); gpos[j] = pos(p.gam[j]); }
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   double t = 0.0;
-  uint64_t tq = tq0;
-  int32_t fired = fired0;
-  // binary32 clock: the day's start state and each continuing round's choice of
-  // this lane, for a resume with the binary64 clock
-  int32_t xday[NC];
-  uint8_t chlog[CLOCK == 2 ? kReplayRounds : 1];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) xday[c] = s.x[c];
-  // more than two rounds a day expected at the start state (a0 > 64): the clock
-  // once per round (below)
-  bool dense = false;
-  if (CLOCK == 2) {
-    float T0[2 * NA - 1], a00;
-    dense = thresholds_f32<NA>(cpos, gpos, cinff, gamf, s.x, T0, a00) && a00 > 64.0f;
-  }
-  for (uint32_t kb = kb0;; kb += 32) {
+  uint64_t tq = 0;
+  int32_t fired = 0;
+  for (uint32_t kb = 0;; kb += 32) {
     if (CLOCK > 0 && kb >= kSpecMaxSteps) return -1;
     // 1. draws of this block
     const uint4 w = philox10(make_uint4((uint32_t)v, (uint32_t)day, kb + (uint32_t)lane, rep), k0, k1);
     const uint64_t j52 = ((((uint64_t)w.y) << 32) | w.x) >> 12;
-    double E = 0.0;
-    float Ef = 0.0f;
-    if (CLOCK == 2) Ef = neglog_f32(j52);
-    else E = neglog_u(j52);
+    const double E = neglog_u(j52);
     const double u2 = uniform_open(w.z, w.w);
     const float u2f = f32_of_q53(((((((uint64_t)w.w) << 32) | w.z) >> 12) << 1) | 1ull);
     // 2. embedded chain
     int32_t x[NC], xs[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) { x[c] = s.x[c]; xs[c] = x[c]; }
-    float a0l = 0.0f;
     int stop_at = 32;
-    if (CLOCK == 2) {
-      // The fixed-point iteration below with the binary32 clock in every round:
-      // the clock after each draw comes from the lanes' current states, and the
-      // first draw that is not a certain continue (a0 = 0, a certain stop, or too
-      // close to call) is the day's end candidate e.  Once no choice of the draws
-      // before e changes, those choices are the chain's, so are the states up to
-      // e and the clock through e: the block is decided without waiting for the
-      // draws after e, which cannot matter.
-      int ch = -3;
-      for (int it = 0; it <= 32; ++it) {
-        prefix_state<NA, 32>(x, ch, lane, xs);
-        float T[2 * NA - 1], a0f;
-        int nc = -2;
-        const bool valid = thresholds_f32<NA>(cpos, gpos, cinff, gamf, xs, T, a0f);
-        if (valid) {
-          nc = choice_count_f32<NA>(T, __fmul_rn(a0f, u2f));
-          if (nc < 0) nc = exact_choice<NA>(cinf, p, xs, u2);
-        }
-        // a dense node-day (many rounds) almost never ends inside a round: settle
-        // every lane's choice first and take the clock once
-        if (dense && it < 32 && __ballot_sync(full, nc != ch)) {
-          ch = nc;
-          continue;
-        }
-        uint64_t sc = valid ? q62_of(fminf(__fdividef(Ef, a0f), 1.5f)) : 0ull;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint64_t y = __shfl_up_sync(full, sc, o);
-          if (lane >= o) sc += y;
-        }
-        const uint64_t sl = tq + sc;
-        const unsigned notcont = __ballot_sync(full, !(valid && sl + margin < kQ62One));
-        const int e = notcont ? __ffs(notcont) - 1 : 32;
-        const unsigned diff = __ballot_sync(full, nc != ch) & (e < 32 ? ((1u << e) - 1u) : full);
-        ch = nc;
-        if (diff != 0u) {
-          if (it == 32) return -1;                  // cannot happen (33 rounds suffice)
-          continue;
-        }
-        if (e < 32) {
-          const unsigned ok = __ballot_sync(full, !valid || sl >= kQ62One + margin);
-          if (!((ok >> e) & 1u)) {                  // too close to call
-            const uint32_t rounds = kb >> 5;
-            if (rounds > (uint32_t)kReplayRounds) return -1;
-            // the binary64 clock's Q62 sum through the earlier rounds, from their
-            // logged choices (every one a continue), then that clock from here on
-            uint64_t tqx = 0;
-            int32_t xr[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) xr[c] = xday[c];
-            for (uint32_t r = 0; r < rounds; ++r) {
-              const uint4 wr = philox10(make_uint4((uint32_t)v, (uint32_t)day, (r << 5) + (uint32_t)lane, rep), k0, k1);
-              const double Er = neglog_u(((((uint64_t)wr.y) << 32) | wr.x) >> 12);
-              const int chr = chlog[r];
-              int32_t xsr[NC];
-              prefix_state<NA, 32>(xr, chr, lane, xsr);
-              double P = 0.0;
-#pragma unroll
-              for (int j = 0; j < NA; ++j) {
-                const double ainf = __dmul_rn(cinf[j], i2d_exact(xsr[2 * j]));
-                const double arec = __dmul_rn(p.gam[j], i2d_exact(xsr[2 * j + 1]));
-                const double A = __dadd_rn(ainf, arec);
-                P = (j == 0) ? A : __dadd_rn(P, A);
-              }
-              const double taur = div_pos(Er, P);
-              tqx += __shfl_sync(full, warp_sum(q62_of_f64(le_nonneg(taur, 1.5) ? taur : 1.5)), 0);
-              int32_t aft[NC];
-#pragma unroll
-              for (int j = 0; j < NA; ++j) {
-                const int dj = ((chr >> 1) == j) ? ((chr & 1) ? -1 : 1) : 0;
-                aft[2 * j] = xsr[2 * j] - dj;
-                aft[2 * j + 1] = xsr[2 * j + 1] + dj;
-              }
-#pragma unroll
-              for (int c = 0; c < NC; ++c) xr[c] = __shfl_sync(full, aft[c], 31);
-            }
-            return ssa_warp_node_day<NA, 1>(p, seed, rep, v, day, phi, 0, s, kb, tqx, fired);
-          }
-#pragma unroll
-          for (int c = 0; c < NC; ++c) s.x[c] = __shfl_sync(full, xs[c], e);
-          return fired + e;
-        }
-        tq = __shfl_sync(full, sl, 31);
-        if ((kb >> 5) < (uint32_t)kReplayRounds) chlog[kb >> 5] = (uint8_t)ch;
-        break;
-      }
-      // the whole block continues: the state after lane 31's draw
-      int32_t after[NC];
-#pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        const int dj = (ch >= 0 && (ch >> 1) == j) ? ((ch & 1) ? -1 : 1) : 0;
-        after[2 * j] = xs[2 * j] - dj;
-        after[2 * j + 1] = xs[2 * j + 1] + dj;
-      }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) s.x[c] = __shfl_sync(full, after[c], 31);
-      fired += 32;
-      continue;
-    }
     if (CLOCK == 1) {
       // Fixed-point iteration over the lanes: every lane takes as its state the
       // block's start plus the transitions currently guessed for the lanes before
@@ -687,7 +782,6 @@ __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_
         float T[2 * NA - 1], a0f;
         int nc = -2;
         if (thresholds_f32<NA>(cpos, gpos, cinff, gamf, xs, T, a0f)) {
-          a0l = a0f;
           nc = spec_ok ? choice_count_f32<NA>(T, __fmul_rn(a0f, u2f)) : -1;
           if (nc < 0) nc = exact_choice<NA>(cinf, p, xs, u2);
         }
@@ -717,7 +811,6 @@ __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_
       float T[2 * NA - 1], a0f;
       const bool any = thresholds_f32<NA>(cpos, gpos, cinff, gamf, x, T, a0f);
       if (!any) { stop_at = l; break; }           // a0 = 0: nothing can fire
-      if (l == lane) a0l = a0f;
       const float ul = __shfl_sync(full, u2f, l);
       int choice = spec_ok ? choice_count_f32<NA>(T, __fmul_rn(a0f, ul)) : -1;
       if (choice < 0) {                            // too close to call: exact arithmetic
@@ -731,25 +824,21 @@ __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_
       }
     }
     int end_at = -1;
-    double tau = 0.0;
-    if (CLOCK < 2) {
-      // 3. exact a0 and tau of each lane's draw
-      double P = 0.0;
+    // 3. exact a0 and tau of each lane's draw
+    double P = 0.0;
 #pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        const double ainf = __dmul_rn(cinf[j], i2d_exact(xs[2 * j]));
-        const double arec = __dmul_rn(p.gam[j], i2d_exact(xs[2 * j + 1]));
-        const double A = __dadd_rn(ainf, arec);
-        P = (j == 0) ? A : __dadd_rn(P, A);
-      }
-      tau = (lane < stop_at && pos(P)) ? div_pos(E, P) : 0.0;
+    for (int j = 0; j < NA; ++j) {
+      const double ainf = __dmul_rn(cinf[j], i2d_exact(xs[2 * j]));
+      const double arec = __dmul_rn(p.gam[j], i2d_exact(xs[2 * j + 1]));
+      const double A = __dadd_rn(ainf, arec);
+      P = (j == 0) ? A : __dadd_rn(P, A);
     }
+    const double tau = (lane < stop_at && pos(P)) ? div_pos(E, P) : 0.0;
     if (CLOCK > 0) {
-      // 4. Q62 scan of tau~ (binary32) or tau (binary64), certain decisions only
+      // 4. Q62 scan of tau, certain decisions only
       const bool valid = lane < stop_at;
-      uint64_t sc = 0ull, m = margin;
-      sc = valid ? q62_of_f64(le_nonneg(tau, 1.5) ? tau : 1.5) : 0ull;
-      m = ((uint64_t)kb + (uint64_t)lane + 2ull) << 10;   // (k + 2) 2^-52
+      uint64_t sc = valid ? q62_of_f64(le_nonneg(tau, 1.5) ? tau : 1.5) : 0ull;
+      const uint64_t m = ((uint64_t)kb + (uint64_t)lane + 2ull) << 10;   // (k + 2) 2^-52
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint64_t y = __shfl_up_sync(full, sc, o);
@@ -794,7 +883,7 @@ __device__ __forceinline__ int32_t ssa_warp_node_day(const DevParams& p, uint64_
 // Group method: the warp's lanes form 32/SEG groups of SEG lanes, one node each
 // (medium herds), with the binary32 clock: per round each group draws SEG steps
 // at once and decides them by the fixed-point iteration of the warp method, with
-// the clock inside every round (CLOCK = 2 above), all groups in lockstep (the
+// the clock inside every round, all groups in lockstep (the
 // warp iterates until every group is decided; a decided group's values stay put,
 // as re-deciding a consistent guess gives the same values).  Every lane returns
 // its group's result: the transitions fired, or -1 (binary32 bounds not met, or a
@@ -978,12 +1067,12 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
       if (active) {                                // warp-uniform
         f = -1;
         if (a.clock_margin) {
-          f = ssa_warp_node_day<NA, 2>(p, a.seed, rep, v, a.day, phi, a.clock_margin, s);
+          f = ssa_warp_day_spec<NA>(p, a.seed, rep, v, a.day, phi, clock_margin_f32(a.clock_margin), s);
           if (f < 0) s = s0;
         }
         if (f < 0) {
-          f = ssa_warp_node_day<NA, 1>(p, a.seed, rep, v, a.day, phi, 0, s);
-          if (f < 0) { s = s0; f = ssa_warp_node_day<NA, 0>(p, a.seed, rep, v, a.day, phi, 0, s); }
+          f = ssa_warp_node_day<NA, 1>(p, a.seed, rep, v, a.day, phi, s);
+          if (f < 0) { s = s0; f = ssa_warp_node_day<NA, 0>(p, a.seed, rep, v, a.day, phi, s); }
         }
       }
     } else {
@@ -1004,8 +1093,8 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
         NodeState<NA> t, t0;
 #pragma unroll
         for (int c = 0; c < 2 * NA; ++c) t.x[c] = t0.x[c] = __shfl_sync(full, s0.x[c], l);
-        int32_t g = ssa_warp_node_day<NA, 1>(p, a.seed, rep, vl, a.day, phil, 0, t);
-        if (g < 0) { t = t0; g = ssa_warp_node_day<NA, 0>(p, a.seed, rep, vl, a.day, phil, 0, t); }
+        int32_t g = ssa_warp_node_day<NA, 1>(p, a.seed, rep, vl, a.day, phil, t);
+        if (g < 0) { t = t0; g = ssa_warp_node_day<NA, 0>(p, a.seed, rep, vl, a.day, phil, t); }
         const bool mine = role == kRoleGroup ? (lane & ~(kGroupLanes - 1)) == l : lane == l;
         if (mine) { s = t; f = g; }
       }
