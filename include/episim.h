@@ -308,9 +308,10 @@ sim_status sim_schedule_events(int32_t n_nodes, int32_t model, int32_t max_days,
 /* Launch shape of the stochastic step.  Nodes whose initial herd has at least
  * warp_herd_threshold animals are simulated one per warp (the 32 lanes draw
  * and time 32 steps at once; suited to herds with many transitions per day);
- * the others one per thread.  -1 = automatic (warps for herds of >= 400 animals
- * while node-replicates number fewer than 152 x 1024, else none); a very large
- * value disables the warp path.  Results do not depend on this setting.  Score
+ * the others one per thread.  -1 = automatic (the largest herds, as many as leave
+ * each unit of work -- a herd per warp, 32 herds per warp -- a resident warp, and
+ * herds whose one-thread day would outlast the whole step); a very large value
+ * disables the warp path.  Results do not depend on this setting.  Score
  * mode always uses one thread per node.  Synchronises the device. */
 sim_status sim_tune(sim_handle* h, int32_t warp_herd_threshold);
 /* Number of nodes currently simulated one per warp (-1 for a NULL handle). */
@@ -320,12 +321,11 @@ int32_t sim_warp_nodes(const sim_handle* h);
  *   SIM_OPT_WARP_THRESHOLD: as sim_tune.
  *   SIM_OPT_GROUP_THRESHOLD: herds below the warp threshold with at least this
  *     many animals (initial herd) are simulated four to a warp, eight lanes each
- *     drawing eight steps at a time; -1 = automatic (200 while node-replicates
- *     number fewer than 152 x 1024, else none), a very large value disables it.
+ *     drawing eight steps at a time; -1 = automatic (none), a very large value
+ *     disables it.
  *   SIM_OPT_CLOCK_MARGIN: k in [0, 17].  The stochastic step (outside score
- *     mode) first runs each node-day with a binary32 clock accumulated in fixed
- *     point, whose distance to the binary64 clock of Eq. (numstep3) is bounded
- *     below 2^-17 of a day; a stop/continue decision within 2^-k of the day's end
+ *     mode) first runs each node-day with a binary32 clock, whose distance to the
+ *     binary64 clock of Eq. (numstep3) is bounded below 2^-17 of a day; a stop/continue decision within 2^-k of the day's end
  *     reruns the node-day with the exact binary64 arithmetic.  k = 17 (default)
  *     is the tightest safe margin; smaller k only reruns more node-days; 0 runs
  *     every node-day exactly.  Values outside [0, 17]: SIM_E_INVALID_ARG.

@@ -76,6 +76,8 @@ struct sim_handle {
   int32_t item_cap = 0;
   long long flow_spin_limit = 1ll << 22;  // ~2 s of polling per wait
   int32_t n_big = 0;                // leading nodes of the order simulated one per warp
+  double animal_rate = 0.0;         // transitions an animal fires a day at the endemic level (endemic_rate)
+  std::vector<int32_t> herd_sorted; // initial herds in the node order (descending)
   int32_t warp_threshold = -1;      // herd size from which a node gets a warp (-1: automatic)
   int32_t group_threshold = -1;     // herd size from which a node gets an 8-lane group (-1: automatic)
   int32_t n_mid = 0;                // nodes after the warp-path ones simulated one per 8-lane group
@@ -348,11 +350,6 @@ SsaArgs ssa_args(sim_handle* h) {
   return a;
 }
 
-// Node order of the stochastic step: nodes with at least `threshold` animals
-// (initial herd) first, one warp each, largest first; then the others, largest
-// first, one thread each (similar work per warp).  threshold < 0: automatic --
-// warps only while the per-thread work leaves the GPU under-occupied (fewer than
-// 152 x 1024 node-replicates), for herds of 400 animals or more.
 // Tables of the split day step: the stochastic step of day d + 1 runs as two
 // launches, the herds that day d's events leave untouched (alongside the event
 // step of day d, on a second stream) and the touched ones (after it).  Per day:
@@ -394,6 +391,65 @@ sim_status build_split(sim_handle* h) {
   return SIM_OK;
 }
 
+// Transitions an animal fires a day at the endemic level of the handle's parameters
+// (mean over replicates and, by initial animals, over classes): S_j -> I_j and back
+// balance at prevalence p, 2 gamma p a day; with phi at (alpha p + eps) / beta the balance
+// upsilon phi (1 - p) = gamma p gives p = 1 - beta gamma / (upsilon alpha) up to eps.
+double endemic_rate(const sim_handle* h) {
+  double class_animals[kMaxAge] = {0.0, 0.0, 0.0}, total = 0.0, phi0 = 0.0, sum = 0.0;
+  for (int c = 0; c < h->nc; ++c)
+    for (int v = 0; v < h->cfg.n_nodes; ++v) class_animals[c / 2] += h->u0[(size_t)c * h->cfg.n_nodes + v];
+  for (double c : class_animals) total += c;
+  if (total <= 0.0) return 0.0;
+  for (double p : h->phi0) phi0 += p;
+  phi0 /= (double)h->phi0.size();
+  for (const DevParams& d : h->params) {
+    double ups = 0.0, gam = 0.0;
+    for (int j = 0; j < h->n_age; ++j) {
+      ups += d.ups[j] * class_animals[j] / total;
+      gam += d.gam[j] * class_animals[j] / total;
+    }
+    const double beta = (d.beta[0] + d.beta[1] + d.beta[2] + d.beta[3]) / 4.0;
+    double p = 0.0;
+    if (beta > 0.0 && ups * d.alpha > 0.0) p = std::max(0.0, 1.0 - beta * gam / (ups * d.alpha));
+    else if (beta == 0.0) p = d.alpha > 0.0 ? 1.0 : (ups * phi0 > 0.0 ? ups * phi0 / (ups * phi0 + gam) : 0.0);
+    sum += 2.0 * gam * p;
+  }
+  return sum / (double)h->params.size();
+}
+
+// Herd size from which a one-thread day would outlast a step of `waves` waves of warps:
+// 25 expected transitions a day per wave.
+int32_t chain_threshold(const sim_handle* h, double waves) {
+  return h->animal_rate > 0.0 ? (int32_t)std::min<double>(1 << 30, 25.0 * std::max(1.0, waves) / h->animal_rate) : 1 << 30;
+}
+
+// Automatic herd size of the warp path (herds sorted, largest first).  While the work
+// units (a herd per warp, then 32 herds per warp) fit one wave of resident warps with a
+// tenth to spare, the largest herds take the spare warps: a warp's node-day takes about
+// as long as a thread's of 20-30 transitions, and nothing waits for the warp.  Beyond one
+// wave a warp unit takes the place of 32 herds, and only herds whose one-thread chain
+// would outlast the launch get one (chain_threshold).
+// Measured, one GB300 (ms a run): national x 365 days 5.5 with 1,007 warp herds (one
+// wave), 7.7 with none, 7.0 with 3,146; 5,000 SISe herds x 200 days 2.8 with 2,249, 3.6
+// with none, 3.3 with 3,753; 16 replicates of the national network at the batched
+// parameters x 100 days, eight waves, 12.2 with 114 warp herds a replicate, 17.6 with
+// none, 14.6 with 697; 64 replicates, persistent, 170 with 4, 175 with none, 183 with 114.
+int32_t auto_threshold(const sim_handle* h) {
+  const int64_t n = (int64_t)h->herd_sorted.size(), R = h->cfg.n_replicates;
+  if (n == 0) return 1 << 30;
+  const int64_t warps = (int64_t)h->sm_count * ssa_resident_warps(h->n_age);
+  const int64_t per = warps * 9 / 10 / R;
+  const int64_t fit = std::min(n, std::max<int64_t>(0, (32 * per - n) / 31));   // fit + (n - fit) / 32 <= per
+  int32_t thr = chain_threshold(h, (double)R * (double)n / 32.0 / (double)warps);
+  // herds of the size of the first one that does not fit stay together
+  if (fit > 0) thr = std::min(thr, fit == n ? 0 : h->herd_sorted[(size_t)fit] + 1);
+  return thr;
+}
+
+// Node order of the stochastic step: nodes with at least `threshold` animals (initial
+// herd) first, one warp each, largest first; then the others, largest first, one thread
+// each (similar work per warp).  threshold < 0: automatic (above).
 sim_status set_order(sim_handle* h, int32_t threshold) {
   const int N = h->cfg.n_nodes;
   std::vector<int64_t> herd(N, 0);
@@ -403,16 +459,11 @@ sim_status set_order(sim_handle* h, int32_t threshold) {
   std::vector<int32_t> order(n_own);
   for (int i = 0; i < n_own; ++i) order[i] = h->node_lo + i;
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return herd[a] > herd[b]; });
-  int32_t thr = threshold;
-  if (thr < 0) {
-    const int64_t work = (int64_t)N * h->cfg.n_replicates;
-    thr = (work < 152 * 1024) ? 400 : (1 << 30);
-  }
-  int32_t gthr = h->group_threshold;
-  if (gthr < 0) {
-    const int64_t work = (int64_t)N * h->cfg.n_replicates;
-    gthr = (work < 152 * 1024) ? 200 : (1 << 30);
-  }
+  h->herd_sorted.resize((size_t)n_own);
+  for (int i = 0; i < n_own; ++i) h->herd_sorted[(size_t)i] = (int32_t)herd[(size_t)order[(size_t)i]];   // <= 2^30
+  h->animal_rate = endemic_rate(h);
+  const int32_t thr = threshold < 0 ? auto_threshold(h) : threshold;
+  const int32_t gthr = h->group_threshold < 0 ? (1 << 30) : h->group_threshold;   // automatic: no group path
   int32_t nb = 0, nm = 0;
   if (!(h->cfg.flags & SIM_FLAG_SCORE)) {
     while (nb < n_own && herd[order[nb]] >= thr) ++nb;
@@ -2061,12 +2112,26 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
   const int smem_limit = batch_min_blocks(shape) > 1 ? (int)(kBatchSmemSM / batch_min_blocks(shape)) : (int)kEventsSmemLimit;
   bool score_any = false;
   const int wpb = threads / 32;
+  // the instances' automatic warp herds were chosen for each alone: together they keep
+  // them while every unit still has a resident warp (chain_threshold otherwise)
+  double units = 0.0;
+  for (int k = 0; k < ni; ++k) {
+    const sim_handle* h = hs[idx[k]];
+    units += (double)h->cfg.n_replicates * (h->n_big + (h->cfg.n_nodes - h->n_big) / 32.0);
+  }
+  const double warps = (double)hs[idx[0]]->sm_count * (threads / 32) * batch_min_blocks(shape);
+  const bool one_wave = units <= 0.9 * warps;
   for (int k = 0; k < ni; ++k) {
     sim_handle* h = hs[idx[k]];
     BatchInst& I = inst[k];
     std::memset(&I, 0, sizeof I);
     I.ssa = ssa_args(h);
-    I.ssa.warp_blocks = (h->n_big + wpb - 1) / wpb;
+    if (h->warp_threshold < 0 && !one_wave) {
+      const int32_t thr = chain_threshold(h, units / warps);
+      I.ssa.n_big = 0;
+      while (I.ssa.n_big < (int32_t)h->herd_sorted.size() && h->herd_sorted[(size_t)I.ssa.n_big] >= thr) ++I.ssa.n_big;
+    }
+    I.ssa.warp_blocks = (I.ssa.n_big + wpb - 1) / wpb;
     I.na = h->n_age;
     I.score = (h->cfg.flags & SIM_FLAG_SCORE) ? 1 : 0;
     if (I.score) { I.ssa.n_big = 0; I.ssa.warp_blocks = 0; }

@@ -193,6 +193,8 @@ struct FinalizeArgs {
   SsaArgs s;                  // day = last simulated day; prologue semantics for day+1
 };
 
+// Warps of the per-day stochastic step an SM holds at once.
+int ssa_resident_warps(int n_age);
 cudaError_t launch_ssa_day(const SsaArgs& a, int n_age, bool score, cudaStream_t st);
 // Region totals of day `day` for every replicate, added (and squared) into s1 / s2
 // [max_days][J][Nc]; the goal terms over count entries of s1 / s2 from `first`.

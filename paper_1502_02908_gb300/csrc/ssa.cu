@@ -32,10 +32,9 @@ __global__ void __launch_bounds__(SCORE ? 256 : 512, SCORE ? (NA == 1 ? 4 : 3) :
   node_day_dealt<NA, SCORE>(a);
 }
 
+// Blocks of 8 warps an SM holds at once.
 template <bool SCORE>
-static cudaError_t launch_dealt(const SsaArgs& a, int n_age, cudaStream_t st) {
-  // resident grid: G = SMs x (blocks of 8 warps an SM holds, fewer when the
-  // units do not fill them); W warps per block, each looping over its units
+static cudaError_t resident_blocks(int n_age, int* out) {
   static int resident[2] = {0, 0};
   const int which = n_age == 1 ? 0 : 1;
   if (!resident[which]) {
@@ -46,12 +45,29 @@ static cudaError_t launch_dealt(const SsaArgs& a, int n_age, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     resident[which] = nb > 0 ? nb : 1;
   }
+  *out = resident[which];
+  return cudaSuccess;
+}
+
+int ssa_resident_warps(int n_age) {
+  int nb = 1;
+  if (resident_blocks<false>(n_age, &nb) != cudaSuccess) return 8;
+  return 8 * nb;
+}
+
+template <bool SCORE>
+static cudaError_t launch_dealt(const SsaArgs& a, int n_age, cudaStream_t st) {
+  // resident grid: G = SMs x (blocks of 8 warps an SM holds, fewer when the
+  // units do not fill them); W warps per block, each looping over its units
+  int resident = 1;
+  const cudaError_t e = resident_blocks<SCORE>(n_age, &resident);
+  if (e != cudaSuccess) return e;
   const int64_t units =
       (int64_t)a.R * (a.n_big + (a.n_mid + 3) / 4 + (a.n_list - a.n_big - a.n_mid + 31) / 32);
   if (units == 0) return cudaSuccess;
   const int64_t sms = a.sm_count > 0 ? a.sm_count : 1;
   const int64_t wmax = a.max_warps > 0 ? a.max_warps : 8;
-  const int64_t fit = a.max_per_sm > 0 ? std::min(resident[which], a.max_per_sm) : resident[which];
+  const int64_t fit = a.max_per_sm > 0 ? std::min(resident, a.max_per_sm) : resident;
   const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(fit, (units + sms * wmax - 1) / (sms * wmax)));
   const int64_t G = sms * per_sm;
   const int W = (int)std::min<int64_t>(wmax, (units + G - 1) / G);
