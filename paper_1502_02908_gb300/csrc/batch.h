@@ -13,7 +13,7 @@ constexpr int batch_min_blocks(BatchShape s) {
   return s == BatchShape::k256x2 ? 2 : s == BatchShape::k128x4 ? 4 : 1;
 }
 constexpr int kBatchTimeout = 2;      // error bit: a bounded wait ran out
-constexpr int kBatchSubs = 4;         // blocks' worth of per-thread nodes in a chunk
+constexpr int kBatchSubs = 4;         // most blocks' worth of per-thread nodes in a chunk
 
 struct BatchInst {
   SsaArgs ssa;            // node order / warp split set for one block's chunks
