@@ -66,11 +66,10 @@ __device__ __forceinline__ double q58_to_double(uint64_t q) {
   return bits_to_double(((uint64_t)e << 52) | (mant & ((1ull << 52) - 1)));
 }
 
-// floor(a * b / 2^62) for signed Q62 operands whose product fits.
-__device__ __forceinline__ int64_t mul_q62(int64_t a, int64_t b) {
-  int64_t hi = __mul64hi(a, b);
-  uint64_t lo = (uint64_t)a * (uint64_t)b;
-  return (int64_t)(((uint64_t)hi << 2) | (lo >> 62));
+// floor(a b / 2^62) for Q62 operands, a given as 4a (|a| < 2^61) and 0 <= b < 2^63: the
+// high half of 4a b, whose unsigned product is too large by b when a is negative.
+__device__ __forceinline__ int64_t mul_q62(int64_t a4, int64_t b) {
+  return (int64_t)(__umul64hi((uint64_t)a4, (uint64_t)b) - ((uint64_t)(a4 >> 63) & (uint64_t)b));
 }
 
 __device__ const int32_t kRecip[128] = {EPISIM_RECIP_TABLE};
@@ -90,14 +89,15 @@ __device__ __forceinline__ double neglog_u(uint64_t j) {
   int i = (int)((M >> 45) & 127);
   int64_t R = __ldg(&kRecip[i]);
   int64_t z = (int64_t)(M * (uint64_t)R) - (int64_t)(1ull << 62);
+  const int64_t z4 = z << 2;
   int64_t h = q62_over(7);
-  h = q62_over(6) - mul_q62(z, h);
-  h = q62_over(5) - mul_q62(z, h);
-  h = q62_over(4) - mul_q62(z, h);
-  h = q62_over(3) - mul_q62(z, h);
-  h = q62_over(2) - mul_q62(z, h);
-  h = q62_over(1) - mul_q62(z, h);
-  int64_t lnm = mul_q62(z, h) + __ldg(&kLogR[i]);
+  h = q62_over(6) - mul_q62(z4, h);
+  h = q62_over(5) - mul_q62(z4, h);
+  h = q62_over(4) - mul_q62(z4, h);
+  h = q62_over(3) - mul_q62(z4, h);
+  h = q62_over(2) - mul_q62(z4, h);
+  h = q62_over(1) - mul_q62(z4, h);
+  int64_t lnm = mul_q62(z4, h) + __ldg(&kLogR[i]);
   // (53 - n) * ln2 in 128 bits minus sign-extended lnm
   uint64_t k = (uint64_t)(53 - n);
   uint64_t p_lo = k * EPISIM_LN2_Q62;

@@ -1,14 +1,14 @@
 // IEEE-754 binary64 division x / y (round to nearest, ties to even) for positive
 // normal operands, on the integer pipe.  On GB300 the FP64 divide takes 562
-// cycles and ~7 FP64 issue slots; this takes ~45 integer instructions.
+// cycles and ~7 FP64 issue slots; this takes ~90 integer instructions.
 //
-// Method (Moller & Granlund, "Improved division by invariant integers", IEEE
-// Trans. Computers 60(2), 2011): the divisor's significand is normalised to a
-// 64-bit d >= 2^63; its reciprocal v = floor((2^128 - 1) / d) - 2^64 comes from
-// an 8-bit table and Newton steps (their Alg. 2); the 128-by-64 quotient of the
-// dividend's significand is their 2-by-1 division with that reciprocal (Alg. 4),
-// which also yields the exact remainder, so the rounding bit and sticky bit are
-// exact.  Subnormal, zero, infinite or NaN operands, and quotients outside the
+// Method: the quotient of the significands as an integer with one guard bit and its
+// exact remainder, so the rounding bit and sticky bit are exact.  On the host, after
+// Moller & Granlund, "Improved division by invariant integers", IEEE Trans. Computers
+// 60(2), 2011: the divisor's significand normalised to a 64-bit d >= 2^63, its
+// reciprocal v = floor((2^128 - 1) / d) - 2^64 by Newton steps (their Alg. 2), the
+// 128-by-64 quotient by their 2-by-1 division (Alg. 4).  On the device, from a
+// binary32 reciprocal and one second-order correction, made exact by the remainder.  Subnormal, zero, infinite or NaN operands, and quotients outside the
 // normal range, take the hardware divide (never the case for the simulation's
 // positive rates and times).  Results are bit-identical to IEEE division.
 #pragma once
@@ -58,28 +58,8 @@ EPI_HD double hw_div(double x, double y) {
 #endif
 }
 
-// v0 of the reciprocal: floor((2^19 - 3 * 2^8) / d9) for d9 = 256..511.  On
-// the device a table built at compile time from the same formula replaces the
-// integer divide.
-struct RecipSeedTable {
-  uint16_t v[256];
-};
-constexpr RecipSeedTable make_recip_seed_table() {
-  RecipSeedTable t{};
-  for (int i = 0; i < 256; ++i) t.v[i] = (uint16_t)(((1u << 19) - 3u * (1u << 8)) / (256u + (unsigned)i));
-  return t;
-}
-#if defined(__CUDACC__)
-__device__ constexpr RecipSeedTable kRecipSeed = make_recip_seed_table();
-#endif
-
-EPI_HD uint64_t recip_seed(uint64_t d9) {
-#if defined(__CUDA_ARCH__)
-  return kRecipSeed.v[d9 - 256u];
-#else
-  return (uint64_t)((1u << 19) - 3u * (1u << 8)) / d9;
-#endif
-}
+// v0 of the reciprocal: floor((2^19 - 3 * 2^8) / d9) for d9 = 256..511.
+EPI_HD uint64_t recip_seed(uint64_t d9) { return (uint64_t)((1u << 19) - 3u * (1u << 8)) / d9; }
 
 // v = floor((2^128 - 1) / d) - 2^64 for 2^63 <= d < 2^64.
 EPI_HD uint64_t recip_u64(uint64_t d) {
@@ -128,8 +108,26 @@ EPI_HD double div_pos(double x, double y) {
   if (e <= 0 || e >= 2047) return hw_div(x, y);   // subnormal or overflowing quotient
   // Q = floor(mx 2^53 / my) = floor(mx 2^64 / (my 2^11)), in [2^53, 2^54)
   const uint64_t d = my << 11;
-  uint64_t rem;
-  const uint64_t Q = div_2by1(mx, 0u, d, recip_u64(d), &rem);
+  uint64_t rem, Q;
+#if defined(__CUDA_ARCH__)
+  // x0 2^-87 = 1 / d to 2^-21 from the binary32 reciprocal of its high word; with f = 1 -
+  // d x0 2^-87, 1 / d = x0 2^-87 (1 + f + f^2 + O(2^-63)): Q to 2^-5, then made exact
+  // by its remainder.  About 60 instructions; the 64-bit reciprocal by table and four
+  // Newton steps of the host's form took about 140.
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint2float_rn((uint32_t)(d >> 32))));
+  const uint32_t x0 = __float2uint_rz(rf * 3.6028797018963968e16f);        // 2^55
+  const int64_t f = (int64_t)(1ull << 62) - (int64_t)((((d >> 32) * x0) << 7) + (((d & 0xffffffffu) * x0) >> 25));   // Q62
+  const int32_t fs = (int32_t)(f >> 18);                                   // Q44
+  const int64_t g = f + (((int64_t)fs * fs) >> 26);
+  const uint64_t q8 = (((mx >> 32) * x0) << 17) + (((mx & 0xffffffffu) * x0) >> 15);   // Q 2^8 to 2^-21, below 2^63
+  Q = (uint64_t)((int64_t)q8 + __mul64hi((int64_t)q8, g << 2)) >> 8;
+  rem = (mx << 53) - Q * my;                                               // mod 2^64: in (-my, 2 my)
+  if ((int64_t)rem < 0) { Q -= 1u; rem += my; }
+  else if (rem >= my) { Q += 1u; rem -= my; }
+#else
+  Q = div_2by1(mx, 0u, d, recip_u64(d), &rem);
+#endif
   uint64_t mant = Q >> 1;                          // 53 bits
   const uint64_t guard = Q & 1u;
   if (guard && (rem != 0u || (mant & 1u))) mant += 1u;

@@ -66,9 +66,10 @@ struct DayTerms {
   double n_inf, n_rec, int_s, int_i, tlast;
 };
 
-// The direct method for one node-day; returns the number of transitions fired.
-template <int NA, bool SCORE>
-__device__ __forceinline__ uint32_t ssa_node_day(const DevParams& p, uint64_t seed, uint32_t rep, int v, int day,
+// The direct method for one node-day with its score terms, in binary64 throughout (nodes
+// outside the bounds of ssa_node_day_score); returns the transitions fired.
+template <int NA>
+__device__ __noinline__ uint32_t ssa_node_day_exact(const DevParams& p, uint64_t seed, uint32_t rep, int v, int day,
                                                  double phi, NodeState<NA>& s, DayTerms (&T)[NA]) {
   double cinf[NA], ainf[NA], arec[NA], A[NA];
 #pragma unroll
@@ -77,7 +78,7 @@ __device__ __forceinline__ uint32_t ssa_node_day(const DevParams& p, uint64_t se
     ainf[j] = __dmul_rn(cinf[j], i2d_exact(s.x[2 * j]));
     arec[j] = __dmul_rn(p.gam[j], i2d_exact(s.x[2 * j + 1]));
     A[j] = __dadd_rn(ainf[j], arec[j]);
-    if (SCORE) { T[j].n_inf = T[j].n_rec = T[j].int_s = T[j].int_i = 0.0; T[j].tlast = 0.0; }
+    { T[j].n_inf = T[j].n_rec = T[j].int_s = T[j].int_i = 0.0; T[j].tlast = 0.0; }
   }
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   double t = 0.0;
@@ -111,7 +112,7 @@ __device__ __forceinline__ uint32_t ssa_node_day(const DevParams& p, uint64_t se
       if (j != cls) continue;
       double thr = (j == 0) ? ainf[0] : __dadd_rn(P[j > 0 ? j - 1 : 0], ainf[j]);
       bool infect = pos(ainf[j]) && (le_nonneg(rr, thr) || !pos(arec[j]));
-      if (SCORE) {
+      {
         double dt = __dsub_rn(t, T[j].tlast);
         T[j].int_s = __dadd_rn(T[j].int_s, __dmul_rn(i2d_exact(s.x[2 * j]), dt));
         T[j].int_i = __dadd_rn(T[j].int_i, __dmul_rn(i2d_exact(s.x[2 * j + 1]), dt));
@@ -126,7 +127,7 @@ __device__ __forceinline__ uint32_t ssa_node_day(const DevParams& p, uint64_t se
     }
     ++fired;
   }
-  if (SCORE) {
+  {
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
       double dt = __dsub_rn(1.0, T[j].tlast);
@@ -340,6 +341,109 @@ __device__ __forceinline__ int exact_choice(const double (&cinf)[NA], const DevP
   return out;
 }
 
+constexpr uint32_t kFastWord = 1u << 20;   // high words from here on stand for their 53-bit uniforms (below)
+
+// Exact binary64 of a non-negative integer below 2^24 held as binary32: five
+// instructions, where the conversion of an int32 (i2d_exact) takes nine.
+__device__ __forceinline__ double f32_count_to_f64(float n) {
+  const uint32_t b = __float_as_uint(n);
+  return __hiloint2double((int)((b >> 3) + (b ? 0x38000000u : 0u)), (int)(b << 29));
+}
+
+// The score's node-day (one thread): the direct method with the specification's own
+// binary64 clock, rates and integrals, whose sums the score terms cancel in, so their
+// every rounding is kept.  Bound by the FP64 pipe (an instruction takes a
+// sub-partition's unit for 64 cycles) and the integer one together: nine binary64
+// operations a step (three for the class's rates, one for the clock, five for the
+// integrals; the plain form has 11), the choice from binary32 rates as in
+// ssa_node_day_spec, counts as binary32 integers, the logarithm and the division on the
+// integer pipe.  (Taking the four products by counts to the integer pipe as well, about
+// 20 instructions each, moved the bound there.)  10,000 SISe herds x 128 replicates x 365
+// days, one GB300: 455 -> 357 ms, 416 with the products on the integer pipe.  False when a
+// herd is too large for binary32 counts or a constant out of their range (s unchanged).
+template <int NA>
+__device__ __forceinline__ bool ssa_node_day_score(const DevParams& p, uint64_t seed, uint32_t rep, int v, int day,
+                                                   double phi, NodeState<NA>& s, DayTerms (&T)[NA], int32_t& fired) {
+  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+  double cinf[NA], A[NA];
+  float cinff[NA], gamf[NA], S[NA], I[NA];
+  int32_t inf[NA], rec[NA];
+#pragma unroll
+  for (int j = 0; j < NA; ++j) cinf[j] = __dmul_rn(p.ups[j], phi);
+  if (!spec_constants<NA>(p, cinf, s.x, cinff, gamf)) return false;
+#pragma unroll
+  for (int j = 0; j < NA; ++j) {
+    S[j] = small_int_to_f32(s.x[2 * j]);
+    I[j] = small_int_to_f32(s.x[2 * j + 1]);
+    A[j] = __dadd_rn(__dmul_rn(cinf[j], f32_count_to_f64(S[j])), __dmul_rn(p.gam[j], f32_count_to_f64(I[j])));
+    T[j].int_s = T[j].int_i = T[j].tlast = 0.0;
+    inf[j] = rec[j] = 0;
+  }
+  double t = 0.0;
+  uint32_t k = 0;
+  for (;; ++k) {
+    double a0 = A[0];
+#pragma unroll
+    for (int j = 1; j < NA; ++j) a0 = __dadd_rn(a0, A[j]);
+    if (!pos(a0)) break;
+    const uint4 w = philox10(make_uint4((uint32_t)v, (uint32_t)day, k, rep), k0, k1);
+    const double E = neglog_u(((((uint64_t)w.y) << 32) | w.x) >> 12);
+    const double tn = __dadd_rn(t, div_pos(E, a0));
+    if (le_nonneg(1.0, tn)) break;
+    t = tn;
+    // selection: the number of thresholds below r~ where every one is at least 64u away
+    float P[2 * NA - 1], a0f = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+      const float ai = __fmul_rn(cinff[j], S[j]);
+      const float Aj = __fmaf_rn(gamf[j], I[j], ai);
+      P[2 * j] = j == 0 ? ai : __fadd_rn(a0f, ai);
+      a0f = j == 0 ? Aj : __fadd_rn(a0f, Aj);
+      if (2 * j + 1 < 2 * NA - 1) P[2 * j + 1 < 2 * NA - 1 ? 2 * j + 1 : 0] = a0f;
+    }
+    const float r = __fmul_rn(a0f, __fmul_rn(__uint2float_rn(w.w), 2.3283064365386963e-10f));
+    float gap = r;
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < 2 * NA - 1; ++i) {
+      const float er = __fsub_rn(r, P[i]);
+      gap = fminf(gap, fabsf(er));
+      c += er > 0.0f ? 1 : 0;
+    }
+    if (w.w < kFastWord || gap < __fmul_rn(r, 3.8146973e-6f)) {
+      int32_t x[2 * NA];
+#pragma unroll
+      for (int j = 0; j < NA; ++j) { x[2 * j] = (int32_t)S[j]; x[2 * j + 1] = (int32_t)I[j]; }
+      c = exact_choice<NA>(cinf, p, x, uniform_open(w.z, w.w));
+    }
+    const float di = (c & 1) ? -1.0f : 1.0f;
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+      if (NA > 1 && (c >> 1) != j) continue;
+      const double dt = __dsub_rn(t, T[j].tlast);
+      T[j].int_s = __dadd_rn(T[j].int_s, __dmul_rn(f32_count_to_f64(S[j]), dt));
+      T[j].int_i = __dadd_rn(T[j].int_i, __dmul_rn(f32_count_to_f64(I[j]), dt));
+      T[j].tlast = t;
+      if (di > 0.0f) ++inf[j]; else ++rec[j];
+      S[j] = __fsub_rn(S[j], di);
+      I[j] = __fadd_rn(I[j], di);
+      A[j] = __dadd_rn(__dmul_rn(cinf[j], f32_count_to_f64(S[j])), __dmul_rn(p.gam[j], f32_count_to_f64(I[j])));
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NA; ++j) {
+    const double dt = __dsub_rn(1.0, T[j].tlast);
+    T[j].int_s = __dadd_rn(T[j].int_s, __dmul_rn(f32_count_to_f64(S[j]), dt));
+    T[j].int_i = __dadd_rn(T[j].int_i, __dmul_rn(f32_count_to_f64(I[j]), dt));
+    T[j].n_inf = i2d_exact(inf[j]);
+    T[j].n_rec = i2d_exact(rec[j]);
+    s.x[2 * j] = (int32_t)S[j];
+    s.x[2 * j + 1] = (int32_t)I[j];
+  }
+  fired = (int32_t)k;
+  return true;
+}
+
 // The direct method for one node-day with the speculative clock (one thread):
 // transitions fired, or -1 when a clock decision was too close to call (the
 // caller then reruns the node-day exactly from the same state).  Bound by issue
@@ -370,7 +474,6 @@ __device__ __forceinline__ int exact_choice(const double (&cinf)[NA], const DevP
 // conversions, a series logarithm, a 64-bit fixed-point clock; about 230
 // instructions a step): 37,000 herds x 64 replicates x 365 days in the persistent
 // kernel 305 -> 172 ms, 1,000 herds x 365 days 7.5 -> 5.7 ms.
-constexpr uint32_t kFastWord = 1u << 20;
 constexpr uint32_t kFastMaxSteps = 1u << 18;   // m's own rounding stays below 2 %
 
 __device__ __forceinline__ float lg2_approx(float x) {
@@ -1057,7 +1160,15 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
       }
       if (SCORE) {
         DayTerms T[NA];
-        f = (int32_t)ssa_node_day<NA, true>(p, a.seed, rep, v, a.day, phi, s, T);
+        if (!ssa_node_day_score<NA>(p, a.seed, rep, v, a.day, phi, s, T, f))
+        {
+          NodeState<NA> se = s;
+          DayTerms Te[NA];
+          f = (int32_t)ssa_node_day_exact<NA>(p, a.seed, rep, v, a.day, phi, se, Te);
+          s = se;
+#pragma unroll
+          for (int j = 0; j < NA; ++j) T[j] = Te[j];
+        }
         accumulate_score<NA>(a, p, r, v, phi, T);
       }
     }

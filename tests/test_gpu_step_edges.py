@@ -88,3 +88,27 @@ def test_step_edges_bitexact(case, tier):
     assert np.array_equal(counts, ref.counts)
     assert np.array_equal(phi, ref.phi)
     assert np.array_equal(ctr, ref.counters)
+
+
+def test_division_at_the_edges_of_its_quotient():
+    # the device division starts from a binary32 reciprocal: quotients just above 1 and
+    # just below 2, divisors that are powers of two or next to one, few-bit operands
+    import torch
+    rng = np.random.default_rng(9)
+    n = 1 << 20
+    one = np.uint64(1) << np.uint64(52)
+    my = rng.integers(0, 1 << 52, n, dtype=np.uint64)
+    my[::4] = rng.integers(0, 4, my[::4].size, dtype=np.uint64)
+    my[1::4] = (1 << 52) - 1 - rng.integers(0, 4, my[1::4].size, dtype=np.uint64)
+    my |= one
+    near = np.uint64(1) << rng.integers(0, 40, n, dtype=np.uint64)
+    mx = np.where(rng.random(n) < 0.5, my + near, 2 * my - near)     # ratio near 1 or near 2
+    ex = np.where(mx >= 2 * one, 1, 0).astype(np.uint64)
+    x = ((np.uint64(1023) + ex) << np.uint64(52)) | ((mx >> ex) & (one - np.uint64(1)))
+    y = (np.uint64(1023) << np.uint64(52)) | (my & (one - np.uint64(1)))
+    xd = torch.from_numpy(x.view(np.float64).copy()).cuda()
+    yd = torch.from_numpy(y.view(np.float64).copy()).cuda()
+    out = torch.empty_like(xd)
+    ref = torch.empty_like(xd)
+    B.debug_div(xd.data_ptr(), yd.data_ptr(), out.data_ptr(), ref.data_ptr(), n, device=True)
+    assert np.array_equal(out.cpu().numpy(), x.view(np.float64) / y.view(np.float64))
