@@ -43,7 +43,13 @@ struct sim_handle {
   int32_t* d_days = nullptr;
   int32_t moments_cap = 0;
   int32_t* d_u0 = nullptr;          // [Nc][N] master copy for resets
-  int32_t* d_order = nullptr;       // node order of the stochastic step
+  int32_t* d_order = nullptr;       // node order of the stochastic step (storage positions)
+  // storage order of the device state: large handles keep their nodes by initial herd,
+  // largest first (permuted()); the host side and the ABI speak of nodes throughout
+  std::vector<int32_t> pos;         // [N] storage position of each node (empty: the node itself)
+  int32_t* d_ids = nullptr;         // [N] node of each position (NULL: the same)
+  unsigned char* d_ws = nullptr;    // staging of state copies into and out of that order
+  size_t ws_bytes = 0;
   int32_t n_order = 0;              // nodes in it: the handle's node range
   int32_t node_lo = 0, node_hi = 0; // nodes whose stochastic step and phi update this handle runs
                                     // (sim_shard; default every node); events apply to all nodes
@@ -251,6 +257,7 @@ void free_all(sim_handle* h) {
   cudaFree(h->d_params); cudaFree(h->d_prev_i);
   cudaFree(h->d_prev_n); cudaFree(h->d_ctr); cudaFree(h->d_err); cudaFree(h->d_score);
   cudaFree(h->d_tang); cudaFree(h->d_u0); cudaFree(h->d_phi0); cudaFree(h->d_order);
+  cudaFree(h->d_ids); cudaFree(h->d_ws);
   cudaFree(h->d_traj); cudaFree(h->d_per_rep); cudaFree(h->d_moments); cudaFree(h->d_days);
   cudaFree(h->d_pack_touched);
   h->d_pack_touched = nullptr;
@@ -262,6 +269,44 @@ void free_all(sim_handle* h) {
 }
 
 bool finite_nonneg(double x) { return std::isfinite(x) && x >= 0.0; }
+
+int32_t at(const sim_handle* h, int32_t node) { return h->pos.empty() ? node : h->pos[(size_t)node]; }
+
+// Copies `planes` planes of N elements (`size` bytes each) between the device state at
+// `dev` and `user` (host or device memory, in node order), through the staging buffer
+// when the state is kept in storage order.  The buffer holds at most kStage bytes (or one
+// plane) whatever the state's size.
+constexpr size_t kStage = (size_t)64 << 20;
+cudaError_t copy_state(sim_handle* h, void* dev, void* user, int64_t planes, int size, bool out, cudaMemcpyKind kind,
+                       cudaStream_t st) {
+  const size_t plane = (size_t)h->cfg.n_nodes * size;
+  if (h->pos.empty())
+    return out ? cudaMemcpyAsync(user, dev, planes * plane, kind, st) : cudaMemcpyAsync(dev, user, planes * plane, kind, st);
+  const int64_t batch = std::min<int64_t>(planes, std::max<int64_t>(1, (int64_t)(kStage / plane)));
+  cudaError_t e = cudaSuccess;
+  if (h->ws_bytes < batch * plane) {
+    e = cudaStreamSynchronize(st);
+    cudaFree(h->d_ws);
+    h->d_ws = nullptr;
+    h->ws_bytes = 0;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_ws, batch * plane);
+    if (e != cudaSuccess) return e;
+    h->ws_bytes = batch * plane;
+  }
+  for (int64_t p = 0; p < planes && e == cudaSuccess; p += batch) {
+    const int64_t n = std::min(batch, planes - p);
+    unsigned char* d = (unsigned char*)dev + p * plane;
+    unsigned char* u = (unsigned char*)user + p * plane;
+    if (out) {
+      e = launch_to_nodes(h->d_ws, d, h->d_ids, h->cfg.n_nodes, n, size, st);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(u, h->d_ws, n * plane, kind, st);
+    } else {
+      e = cudaMemcpyAsync(h->d_ws, u, n * plane, kind, st);
+      if (e == cudaSuccess) e = launch_from_nodes(d, h->d_ws, h->d_ids, h->cfg.n_nodes, n, size, st);
+    }
+  }
+  return e;
+}
 
 size_t n_counts(const sim_handle* h) { return (size_t)h->cfg.n_replicates * h->nc * h->cfg.n_nodes; }
 size_t n_phi(const sim_handle* h) { return (size_t)h->cfg.n_replicates * h->cfg.n_nodes; }
@@ -337,6 +382,7 @@ SsaArgs ssa_args(sim_handle* h) {
   a.pre_event = (h->cfg.flags & SIM_FLAG_PHI_PRE_EVENT) ? 1 : 0;
   a.traj = h->d_traj;
   a.order = h->d_order;
+  a.ids = h->d_ids;
   a.n_big = h->n_big;
   a.n_mid = h->n_mid;
   a.warp_blocks = (h->n_big + 7) / 8;
@@ -373,13 +419,14 @@ sim_status build_split(sim_handle* h) {
     const int32_t b = h->day_touch_host[(size_t)d], e = h->day_touch_host[(size_t)d + 1];
     for (int32_t i = b; i < e; ++i) {
       const int v = h->touched_host[(size_t)i];
-      skip[(size_t)d * words + (size_t)(v >> 5)] |= 1u << (v & 31);
+      skip[(size_t)d * words + (size_t)(at(h, v) >> 5)] |= 1u << (at(h, v) & 31);
       tl[(size_t)i] = v;
     }
     std::stable_sort(tl.begin() + b, tl.begin() + e, [&](int32_t x, int32_t y) { return herd[x] > herd[y]; });
     int32_t nb = 0, nm = 0;
     while (b + nb < e && herd[tl[(size_t)(b + nb)]] >= h->eff_threshold) ++nb;
     while (b + nb + nm < e && herd[tl[(size_t)(b + nb + nm)]] >= h->eff_group_threshold) ++nm;
+    for (int32_t i = b; i < e; ++i) tl[(size_t)i] = at(h, tl[(size_t)i]);
     h->tlist_nbig[(size_t)d] = nb;
     h->tlist_nmid[(size_t)d] = nm;
   }
@@ -470,8 +517,10 @@ sim_status set_order(sim_handle* h, int32_t threshold) {
     while (nb + nm < n_own && herd[order[nb + nm]] >= gthr) ++nm;
   }
   if (!h->d_order) CK(h, dalloc(&h->d_order, (size_t)N), "node order allocation");
+  std::vector<int32_t> where((size_t)n_own);
+  for (int i = 0; i < n_own; ++i) where[(size_t)i] = at(h, order[(size_t)i]);
   if (n_own > 0)
-    CK(h, cudaMemcpy(h->d_order, order.data(), (size_t)n_own * 4, cudaMemcpyHostToDevice), "node order upload");
+    CK(h, cudaMemcpy(h->d_order, where.data(), (size_t)n_own * 4, cudaMemcpyHostToDevice), "node order upload");
   h->n_order = n_own;
   h->order_host.swap(order);
   free_flow(h);
@@ -1148,6 +1197,30 @@ sim_status create_impl(const sim_config* cfg, const int32_t* u0, const double* p
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     h->sm_count = sms > 0 ? sms : 1;
   }
+  // Storage order.  A unit's 32 herds are neighbours in herd size; with the state in that
+  // order too their loads and stores are contiguous instead of one 32-byte sector each.
+  // Worth it once the replicates' state no longer sits close to the SMs: ten national
+  // replicates 68 -> 40 us a day, 64 in the persistent kernel 475 -> 423, one 14.7 -> 14.1
+  // (one GB300); below 2^15 node-replicates, in the caller's buffers and in score mode
+  // (whose sums run over the nodes in order) the nodes stay as they are.
+  if (!dev_counts && !(h->cfg.flags & SIM_FLAG_SCORE) && (int64_t)N * R >= ((int64_t)1 << 15)) {
+    try {
+      std::vector<int64_t> herd((size_t)N, 0);
+      for (int c = 0; c < h->nc; ++c)
+        for (int v = 0; v < N; ++v) herd[(size_t)v] += h->u0[(size_t)c * N + v];
+      std::vector<int32_t> ids((size_t)N);
+      for (int v = 0; v < N; ++v) ids[(size_t)v] = v;
+      std::stable_sort(ids.begin(), ids.end(), [&](int32_t a, int32_t b) { return herd[(size_t)a] > herd[(size_t)b]; });
+      h->pos.resize((size_t)N);
+      for (int i = 0; i < N; ++i) h->pos[(size_t)ids[(size_t)i]] = i;
+      if (e == cudaSuccess) e = dalloc(&h->d_ids, (size_t)N);
+      if (e == cudaSuccess) e = cudaMemcpy(h->d_ids, ids.data(), (size_t)N * 4, cudaMemcpyHostToDevice);
+    } catch (...) {
+      free_all(h);
+      delete h;
+      return fail(nullptr, SIM_E_OOM, "host allocation");
+    }
+  }
   const size_t stats = (size_t)R * (cfg->max_days > 0 ? cfg->max_days : 1);
   if (dev_counts) {
     h->owns_state = false;
@@ -1172,8 +1245,8 @@ sim_status create_impl(const sim_config* cfg, const int32_t* u0, const double* p
   if (e == cudaSuccess && (h->cfg.flags & SIM_FLAG_SCORE_REVERSE))
     e = dalloc(&h->d_traj, (size_t)3 * (cfg->max_days > 0 ? cfg->max_days : 1) * n_phi(h));
   if (e == cudaSuccess) e = cudaMemcpy(h->d_params, h->params.data(), R * sizeof(DevParams), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_u0, h->u0.data(), h->u0.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_phi0, h->phi0.data(), h->phi0.size() * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = copy_state(h, h->d_u0, h->u0.data(), h->nc, 4, false, cudaMemcpyHostToDevice, 0);
+  if (e == cudaSuccess) e = copy_state(h, h->d_phi0, h->phi0.data(), 1, 8, false, cudaMemcpyHostToDevice, 0);
   if (e != cudaSuccess) {
     sim_status s = cuda_fail(nullptr, e, "device allocation / upload");
     free_all(h);
@@ -1216,6 +1289,14 @@ sim_status sim_load_events(sim_handle* h, int64_t n, const int32_t* day, const i
   free_events(h);
   const int32_t T = h->cfg.max_days;
   cudaError_t err = cudaSuccess;
+  std::vector<int32_t> touched;                    // the device's tables name storage positions
+  if (!h->pos.empty()) {
+    try { touched = S.touched; } catch (...) { return fail(h, SIM_E_OOM, "host allocation"); }
+    for (int4& r : S.rec) { r.x = at(h, r.x); if (r.y >= 0) r.y = at(h, r.y); }
+    for (int32_t& v : touched) v = at(h, v);
+    for (int32_t& v : S.touched_df) v = at(h, v);
+  }
+  const std::vector<int32_t>& touched_at = h->pos.empty() ? S.touched : touched;
   if (err == cudaSuccess) err = dalloc(&h->d_rec, S.rec.size());
   if (err == cudaSuccess) err = dalloc(&h->d_lvl_start, S.lvl_start.size());
   if (err == cudaSuccess) err = dalloc(&h->d_day_lvl, (size_t)T + 1);
@@ -1226,7 +1307,7 @@ sim_status sim_load_events(sim_handle* h, int64_t n, const int32_t* day, const i
   if (err == cudaSuccess) err = dalloc(&h->d_touched, S.touched.size());
   if (err == cudaSuccess) err = dalloc(&h->d_day_touch, S.day_touch.size());
   if (err == cudaSuccess && !S.rec_slot.empty()) err = cudaMemcpy(h->d_rec_slot, S.rec_slot.data(), S.rec_slot.size() * sizeof(int4), cudaMemcpyHostToDevice);
-  if (err == cudaSuccess && !S.touched.empty()) err = cudaMemcpy(h->d_touched, S.touched.data(), S.touched.size() * 4, cudaMemcpyHostToDevice);
+  if (err == cudaSuccess && !S.touched.empty()) err = cudaMemcpy(h->d_touched, touched_at.data(), touched_at.size() * 4, cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMemcpy(h->d_day_touch, S.day_touch.data(), S.day_touch.size() * 4, cudaMemcpyHostToDevice);
   if (err != cudaSuccess) { free_events(h); return cuda_fail(h, err, "event upload"); }
   {
@@ -1552,6 +1633,7 @@ static sim_status build_flow(sim_handle* h) {
     if (err == cudaSuccess) err = dalloc(dst, std::max<size_t>(v.size(), 1));
     if (err == cudaSuccess && !v.empty()) err = cudaMemcpy(*dst, v.data(), v.size() * elem, cudaMemcpyHostToDevice);
   };
+  for (int32_t& v : cnode) v = at(h, v);
   up(&h->d_fl_rec, rec, sizeof(int4));
   up(&h->d_fl_cev, cev, 4);
   up(&h->d_fl_cnode, cnode, 4);
@@ -1810,7 +1892,8 @@ sim_status sim_unpack_touched(sim_handle* h, const int32_t* dev_in, int32_t worl
   CK(h, cudaMemcpy(h->d_pack_touched, bounds, ((size_t)world + 1) * 4, cudaMemcpyHostToDevice), "bounds upload");
   const int32_t b = h->day_touch_host[(size_t)h->day];
   CK(h, launch_unpack_touched(h->d_counts, h->d_touched + b, n_t, h->cfg.n_nodes,
-                              (int64_t)h->cfg.n_replicates * h->nc, dev_in, h->d_pack_touched, world, st),
+                              (int64_t)h->cfg.n_replicates * h->nc, dev_in, h->d_pack_touched, world,
+                              h->d_ids, st),
      "unpack launch");
   return SIM_OK;
 }
@@ -1822,8 +1905,8 @@ sim_status sim_state(sim_handle* h, int32_t* counts, double* phi, int32_t* day, 
   if (where != SIM_HOST && where != SIM_DEVICE) return fail(h, SIM_E_INVALID_ARG, "where must be SIM_HOST or SIM_DEVICE");
   cudaStream_t st = (cudaStream_t)stream;
   const cudaMemcpyKind k = where == SIM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-  if (counts) CK(h, cudaMemcpyAsync(counts, h->d_counts, n_counts(h) * 4, k, st), "copy counts");
-  if (phi) CK(h, cudaMemcpyAsync(phi, h->d_phi, n_phi(h) * 8, k, st), "copy phi");
+  if (counts) CK(h, copy_state(h, h->d_counts, counts, (int64_t)h->cfg.n_replicates * h->nc, 4, true, k, st), "copy counts");
+  if (phi) CK(h, copy_state(h, h->d_phi, phi, h->cfg.n_replicates, 8, true, k, st), "copy phi");
   CK(h, cudaStreamSynchronize(st), "stream synchronize");
   if (day) *day = h->day;
   return check_latched(h);
@@ -1843,8 +1926,9 @@ sim_status sim_set_state(sim_handle* h, const int32_t* counts, const double* phi
   }
   cudaStream_t st = (cudaStream_t)stream;
   const cudaMemcpyKind k = where == SIM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-  CK(h, cudaMemcpyAsync(h->d_counts, counts, n_counts(h) * 4, k, st), "copy counts");
-  CK(h, cudaMemcpyAsync(h->d_phi, phi, n_phi(h) * 8, k, st), "copy phi");
+  CK(h, copy_state(h, h->d_counts, const_cast<int32_t*>(counts), (int64_t)h->cfg.n_replicates * h->nc, 4, false, k, st),
+     "copy counts");
+  CK(h, copy_state(h, h->d_phi, const_cast<double*>(phi), h->cfg.n_replicates, 8, false, k, st), "copy phi");
   const int T = h->cfg.max_days;
   if (T > day) {
     const size_t w = (size_t)(T - day) * 8, pitch = (size_t)T * 8;
@@ -1992,7 +2076,9 @@ sim_status sim_set_regions(sim_handle* h, const int32_t* region_of_node, int32_t
   for (int32_t j = 0; j < n_regions; ++j) off[(size_t)j + 1] += off[(size_t)j];
   {
     std::vector<int32_t> fill(off.begin(), off.end() - 1);
-    for (int v = 0; v < N; ++v) nodes[(size_t)fill[(size_t)region_of_node[v]]++] = v;
+    for (int v = 0; v < N; ++v) nodes[(size_t)fill[(size_t)region_of_node[v]]++] = at(h, v);
+    for (int32_t j = 0; j < n_regions; ++j)
+      std::sort(nodes.begin() + off[(size_t)j], nodes.begin() + off[(size_t)j + 1]);   // neighbours in storage together
   }
   const size_t rows = (size_t)std::max(1, h->cfg.max_days) * n_regions * h->nc;
   cudaError_t e = dalloc(&h->d_reg_nodes, nodes.size());

@@ -44,7 +44,9 @@ struct SsaArgs {
   int32_t prologue;           // 1: first record stats of day-1 and (post-event mode) update phi
   int32_t pre_event;          // 1: phi update from post-SSA counts in the epilogue
   double* traj;               // reverse-mode score: [3][max_days][R][N] = c_d, phi_d, I_d/N_d (NULL otherwise)
-  const int32_t* order;       // node order: first n_big nodes warp-cooperative, the rest per thread (NULL: identity)
+  const int32_t* order;       // node order: first n_big nodes warp-cooperative, the rest per thread (NULL: identity).
+                              // Nodes are storage positions here, as in every array the kernels read.
+  const int32_t* ids;         // [N] node of each storage position, for the random counters (NULL: the same)
   int32_t n_list;             // nodes in the order list (N, or a day's touched list)
   const uint32_t* skip;       // bitmap [N] of nodes this launch leaves out (NULL: none)
   int32_t n_big;              // nodes simulated one per warp
@@ -210,7 +212,14 @@ cudaError_t launch_finalize(const SsaArgs& a, int n_age, bool score, cudaStream_
 cudaError_t launch_pack_touched(const int32_t* counts, const int32_t* touched, int n_t, int N, int64_t planes,
                                 int32_t* out, cudaStream_t st);
 cudaError_t launch_unpack_touched(int32_t* counts, const int32_t* touched, int n_t, int N, int64_t planes,
-                                  const int32_t* in, const int32_t* bounds, int world, cudaStream_t st);
+                                  const int32_t* in, const int32_t* bounds, int world, const int32_t* ids,
+                                  cudaStream_t st);
+// Storage order of `planes` planes of N elements of `size` (4 or 8) bytes: to node order
+// (out[ids[i]] = in[i]) or from it (out[i] = in[ids[i]]).
+cudaError_t launch_to_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
+                            cudaStream_t st);
+cudaError_t launch_from_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
+                              cudaStream_t st);
 cudaError_t launch_debug_neglog(const uint64_t* j, double* out, int64_t n, cudaStream_t st);
 cudaError_t launch_debug_neglog_f32(const uint64_t* j, float* out, int64_t n, cudaStream_t st);
 

@@ -1132,6 +1132,7 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
   const bool owner = role == kRoleThread || (role == kRoleWarp ? lane == 0 : (lane & (kGroupLanes - 1)) == 0);
   const DevParams& p = a.params[r];
   const uint32_t rep = (uint32_t)(a.rep_base + r);
+  const int id = MODE == 0 && a.ids ? __ldg(a.ids + v) : v;   // v is the storage position
   double* phip = a.phi + (size_t)r * a.N + v;
   NodeState<NA> s, s0;
   double phi = 0.0;
@@ -1155,16 +1156,16 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
 #pragma unroll
         for (int j = 0; j < NA; ++j) cinf[j] = __dmul_rn(p.ups[j], phi);
         if (spec_constants<NA>(p, cinf, s.x, cinff, gamf)) {
-          f = ssa_node_day_spec<NA>(p, a.seed, rep, v, a.day, cinf, cinff, gamf, clock_margin_f32(a.clock_margin), s);
+          f = ssa_node_day_spec<NA>(p, a.seed, rep, id, a.day, cinf, cinff, gamf, clock_margin_f32(a.clock_margin), s);
         }
       }
       if (SCORE) {
         DayTerms T[NA];
-        if (!ssa_node_day_score<NA>(p, a.seed, rep, v, a.day, phi, s, T, f))
+        if (!ssa_node_day_score<NA>(p, a.seed, rep, id, a.day, phi, s, T, f))
         {
           NodeState<NA> se = s;
           DayTerms Te[NA];
-          f = (int32_t)ssa_node_day_exact<NA>(p, a.seed, rep, v, a.day, phi, se, Te);
+          f = (int32_t)ssa_node_day_exact<NA>(p, a.seed, rep, id, a.day, phi, se, Te);
           s = se;
 #pragma unroll
           for (int j = 0; j < NA; ++j) T[j] = Te[j];
@@ -1178,17 +1179,17 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
       if (active) {                                // warp-uniform
         f = -1;
         if (a.clock_margin) {
-          f = ssa_warp_day_spec<NA>(p, a.seed, rep, v, a.day, phi, clock_margin_f32(a.clock_margin), s);
+          f = ssa_warp_day_spec<NA>(p, a.seed, rep, id, a.day, phi, clock_margin_f32(a.clock_margin), s);
           if (f < 0) s = s0;
         }
         if (f < 0) {
-          f = ssa_warp_node_day<NA, 1>(p, a.seed, rep, v, a.day, phi, s);
-          if (f < 0) { s = s0; f = ssa_warp_node_day<NA, 0>(p, a.seed, rep, v, a.day, phi, s); }
+          f = ssa_warp_node_day<NA, 1>(p, a.seed, rep, id, a.day, phi, s);
+          if (f < 0) { s = s0; f = ssa_warp_node_day<NA, 0>(p, a.seed, rep, id, a.day, phi, s); }
         }
       }
     } else {
       if (role == kRoleGroup) {                    // every lane of the warp takes part
-        f = a.clock_margin ? ssa_seg_node_day<NA, kGroupLanes>(p, a.seed, rep, v, a.day, phi, a.clock_margin,
+        f = a.clock_margin ? ssa_seg_node_day<NA, kGroupLanes>(p, a.seed, rep, id, a.day, phi, a.clock_margin,
                                                                active, s)
                            : (active ? -1 : 0);
         if (f < 0) s = s0;
@@ -1199,7 +1200,7 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
       while (need) {
         const int l = __ffs(need) - 1;
         need &= need - 1;
-        const int vl = __shfl_sync(full, v, l);
+        const int vl = __shfl_sync(full, id, l);
         const double phil = __shfl_sync(full, phi, l);
         NodeState<NA> t, t0;
 #pragma unroll
@@ -1250,6 +1251,9 @@ __device__ __forceinline__ void node_day_block(const SsaArgs& a, int r, int bx) 
     if (MODE == 0 && !SCORE && a.order) {
       active = a.n_big + i < a.n_list;
       v = active ? a.order[a.n_big + i] : 0;
+    } else if (MODE == 1 && a.ids) {               // the handle's nodes, in storage order
+      active = i < a.n_list;
+      v = active ? a.order[i] : 0;
     } else {                                       // the handle's node range, in id order
       v = a.node_lo + i;
       active = v < a.node_hi;
@@ -1279,27 +1283,16 @@ __device__ __forceinline__ void node_day_dealt(const SsaArgs& a) {
   const int64_t ntu = (a.n_list - a.n_big - a.n_mid + 31) / 32;      // 32 nodes per warp
   const int64_t units = uw + ug + R * ntu;
   for (int64_t u = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < units; u += T) {
-    int r = 0, v = 0, role = kRoleThread;
-    bool active = false;
-    if (u < uw) {
-      r = (int)(u % R);
-      v = a.order[u / R];
-      active = true;
-      role = kRoleWarp;
-    } else if (u < uw + ug) {
-      const int64_t ut = u - uw;
-      r = (int)(ut % R);
-      const int64_t i = a.n_big + (ut / R) * 4 + (lane / kGroupLanes);
-      active = i < a.n_big + a.n_mid;
-      v = active ? a.order[i] : 0;
-      role = kRoleGroup;
-    } else {
-      const int64_t ut = u - uw - ug;
-      r = (int)(ut % R);
-      const int64_t i = a.n_big + a.n_mid + (ut / R) * 32 + lane;
-      active = i < a.n_list;
-      v = active ? a.order[i] : 0;
-    }
+    const int role = u < uw ? kRoleWarp : (u < uw + ug ? kRoleGroup : kRoleThread);
+    const int64_t ut = u - (role == kRoleWarp ? 0 : (role == kRoleGroup ? uw : uw + ug));
+    // node group and replicate of the unit (a 32-bit division where it fits)
+    const int64_t gi = R == 1 ? ut : (units < (1ll << 31) ? (int64_t)((uint32_t)ut / (uint32_t)R) : ut / R);
+    const int r = (int)(ut - gi * R);
+    const int64_t i = role == kRoleWarp ? gi
+                                        : (role == kRoleGroup ? a.n_big + gi * 4 + lane / kGroupLanes
+                                                              : a.n_big + a.n_mid + gi * 32 + lane);
+    bool active = role == kRoleWarp || i < (role == kRoleGroup ? a.n_big + a.n_mid : a.n_list);
+    const int v = active ? a.order[i] : 0;
     if (a.skip && active && ((__ldg(a.skip + (v >> 5)) >> (v & 31)) & 1u)) active = false;
     node_day_work<NA, SCORE, 0>(a, r, v, active, role);
   }
