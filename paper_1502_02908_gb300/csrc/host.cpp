@@ -104,6 +104,8 @@ struct sim_handle {
   int32_t n_regions = 0;
   int32_t* d_reg_nodes = nullptr;      // nodes sorted by region
   int32_t* d_reg_off = nullptr;        // [J + 1]
+  int32_t* d_reg_of = nullptr;         // [N] region of each storage position (slab sums; NULL: not used)
+  unsigned long long* d_reg_tot = nullptr;  // [R][J][Nc] totals of the day being summed, then [R] tickets
   unsigned long long* d_s1 = nullptr;  // [max_days][J][Nc]
   unsigned long long* d_s2 = nullptr;
   long long* d_ref = nullptr;          // scratch for sim_goal
@@ -238,7 +240,8 @@ void free_graph(sim_handle* h) {
 
 void free_regions(sim_handle* h) {
   cudaFree(h->d_reg_nodes); cudaFree(h->d_reg_off); cudaFree(h->d_s1); cudaFree(h->d_s2);
-  cudaFree(h->d_ref); cudaFree(h->d_goal);
+  cudaFree(h->d_ref); cudaFree(h->d_goal); cudaFree(h->d_reg_of); cudaFree(h->d_reg_tot);
+  h->d_reg_of = nullptr; h->d_reg_tot = nullptr;
   h->d_reg_nodes = h->d_reg_off = nullptr; h->d_s1 = h->d_s2 = nullptr; h->d_ref = nullptr; h->d_goal = nullptr;
   h->n_regions = 0; h->ref_cap = 0;
 }
@@ -1503,8 +1506,13 @@ static sim_status enqueue_days(sim_handle* h, int32_t d0, int32_t ndays, cudaStr
       if (es != SIM_OK) return es;
     }
     if (h->n_regions > 0)                            // region totals of the state after day d
-      CK(h, launch_region_day(h->d_counts, h->d_reg_nodes, h->d_reg_off, h->cfg.n_nodes, h->cfg.n_replicates,
-                              h->nc, h->n_regions, d, h->d_s1, h->d_s2, st), "region statistics launch");
+      CK(h, h->d_reg_of
+                ? launch_region_slab(h->d_counts, h->d_reg_of, h->cfg.n_nodes, h->cfg.n_replicates, h->nc, h->n_regions,
+                                     d, h->sm_count, h->d_reg_tot,
+                                     (unsigned*)(h->d_reg_tot + (size_t)h->cfg.n_replicates * h->n_regions * h->nc),
+                                     h->d_s1, h->d_s2, st)
+                : launch_region_day(h->d_counts, h->d_reg_nodes, h->d_reg_off, h->cfg.n_nodes, h->cfg.n_replicates,
+                                    h->nc, h->n_regions, d, h->d_s1, h->d_s2, st), "region statistics launch");
   }
   a.day = d0 + ndays - 1;
   CK(h, traced(h, 2, st, [&] { return launch_finalize(a, h->n_age, score, st); }), "phi update launch");
@@ -2090,6 +2098,15 @@ sim_status sim_set_regions(sim_handle* h, const int32_t* region_of_node, int32_t
   if (e == cudaSuccess) e = cudaMemcpy(h->d_reg_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(h->d_s1, 0, rows * 8);
   if (e == cudaSuccess) e = cudaMemset(h->d_s2, 0, rows * 8);
+  if (e == cudaSuccess && region_slab_fits(n_regions, h->nc) && h->cfg.n_replicates <= 65535) {
+    std::vector<int32_t> region_at((size_t)N);
+    for (int v = 0; v < N; ++v) region_at[(size_t)at(h, v)] = region_of_node[v];
+    const size_t tot = (size_t)h->cfg.n_replicates * ((size_t)n_regions * h->nc + 1);
+    e = dalloc(&h->d_reg_of, (size_t)N);
+    if (e == cudaSuccess) e = dalloc(&h->d_reg_tot, tot);
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_reg_of, region_at.data(), (size_t)N * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(h->d_reg_tot, 0, tot * 8);
+  }
   if (e != cudaSuccess) { free_regions(h); return cuda_fail(h, e, "region statistics"); }
   h->n_regions = n_regions;
   return SIM_OK;

@@ -203,6 +203,12 @@ cudaError_t launch_ssa_day(const SsaArgs& a, int n_age, bool score, cudaStream_t
 cudaError_t launch_region_day(const int32_t* counts, const int32_t* reg_nodes, const int32_t* reg_off, int N, int R,
                               int Nc, int J, int day, unsigned long long* s1, unsigned long long* s2,
                               cudaStream_t st);
+// The same from slabs of consecutive nodes, when the block's table fits (region_slab_fits)
+// and R <= 65,535: region_of [N] by storage position; tot [R][J][Nc] and ticket [R] cleared.
+bool region_slab_fits(int J, int Nc);
+cudaError_t launch_region_slab(const int32_t* counts, const int32_t* region_of, int N, int R, int Nc, int J, int day,
+                               int sms, unsigned long long* tot, unsigned* ticket, unsigned long long* s1,
+                               unsigned long long* s2, cudaStream_t st);
 cudaError_t launch_goal(const unsigned long long* s1, const unsigned long long* s2, const long long* ref,
                         long long first, long long count, int R, double* out, cudaStream_t st);
 cudaError_t launch_events_day(const EvArgs& a, int n_age, cudaStream_t st);

@@ -148,3 +148,29 @@ def test_pre_event_phi():
     for x, y in zip(a.state(), b.state()):
         assert np.array_equal(x, y)
     a.close(); b.close()
+
+@pytest.mark.parametrize("J", [1, 7, 683])         # 683 x 6 x 8 bytes: past the slab table, region by region
+def test_region_sums_of_large_herds(J):
+    # slab sums add the low and high 16 bits of a count apart; one node of 2^29 animals
+    w = W.sise3_national(N=5000, T=3, n_events=600, R=2)
+    u0 = w.u0.copy()
+    u0[4, 17] = 1 << 29
+    u0[0, 4999] = (1 << 16) + 3
+    import dataclasses
+    w = dataclasses.replace(w, u0=u0)
+    region = (np.arange(w.N) * 37) % J
+    s = B.Sim.from_workload(w)
+    s.set_regions(region, J)
+    s1 = np.zeros((w.T, J, 6), np.uint64)
+    s2 = np.zeros((w.T, J, 6), np.uint64)
+    for d in range(w.T):
+        s.run(1)
+        counts = s.state()[0].astype(np.uint64)
+        for r in range(w.R):
+            tot = np.stack([np.bincount(region, weights=counts[r, c].astype(np.float64), minlength=J) for c in range(6)], 1)
+            tot = tot.astype(np.uint64)
+            s1[d] += tot
+            s2[d] += tot * tot
+    a, b = s.region_moments()
+    s.close()
+    assert np.array_equal(a, s1) and np.array_equal(b, s2)
