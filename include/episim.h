@@ -407,7 +407,9 @@ sim_status sim_run_batch(sim_handle** handles, int32_t n, const int32_t* until, 
  * needs more than 220 KB / blocks_per_sm runs the global-memory variant.  More
  * resident blocks hide more of the stochastic step's latency at a register budget
  * of 65,536 / (threads x blocks_per_sm) a thread.  Results do not depend on the
- * shape (every random number is keyed by node, day and event position).  The
+ * shape (every random number is keyed by node, day and event position).  With the
+ * default shape a run whose per-thread nodes would not fill its blocks takes one block
+ * an SM.  The
  * paper has no counterpart: this is a launch-tuning knob.  Errors:
  * SIM_E_INVALID_ARG for any other shape. */
 sim_status sim_batch_shape(int32_t threads, int32_t blocks_per_sm);

@@ -12,6 +12,7 @@ CSRC = HERE / "csrc"
 BUILD = HERE / "_build"
 LIB = BUILD / "libepisim.so"
 SOURCES = ["ssa.cu", "events.cu", "batch.cu", "batch_shape_256x1.cu", "batch_shape_256x2.cu", "batch_shape_128x4.cu",
+           "batch_lists_256x1.cu", "batch_lists_256x2.cu",
            "noalloc.cu", "regions.cu", "general.cu", "peak.cu", "shard.cu", "flow.cu", "host.cpp",
            "general_host.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

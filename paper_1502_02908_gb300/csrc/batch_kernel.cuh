@@ -108,10 +108,55 @@ __device__ __forceinline__ void dispatch_chunk(const BatchInst& I, int r, int ch
   }
 }
 
-__device__ __forceinline__ void dispatch_events(const BatchInst& I, int r, int day, unsigned char* smem, int smem_cap) {
+// Part `part` of a day's events by owner lists: a component's events are one thread's
+// list in input order, so a lane applies it straight to the counts, with no levels, no
+// barrier and no staging.  The lists of an owner-computes block go to kBatchEvLanes lanes.
+// Bound by the longest list's chain (about 1,200 cycles an event); the staged step takes
+// one block through every level of the day: 7,972 herds, 1,747 events a day, one GB300:
+// 22 us a day staged, 5 in five parts.
+template <int NA>
+__device__ __forceinline__ void events_by_lists(const BatchInst& I, int r, int day, int part) {
+  const int2 D = __ldg(I.day_df + day);
+  EvArgs a = I.evg;
+  a.day = day;
+  int32_t* X = a.counts + (size_t)r * a.Nc * a.N;
+  unsigned applied = 0, clamped = 0, skipped = 0;
+  const int sub = threadIdx.x % kBatchEvLanes, per = (int)blockDim.x / kBatchEvLanes;
+  for (int b = part * per + (int)threadIdx.x / kBatchEvLanes; b < D.y; b += I.ev_parts * per) {
+    const int4 m0 = __ldg(I.df_meta + D.x + b), m1 = __ldg(I.df_meta + D.x + b + 1);
+    const int lists = m1.z - m0.z - 1;
+    for (int i = sub; i < lists; i += kBatchEvLanes) {
+      const int q1 = __ldg(I.df_thr_off + m0.z + i + 1);
+      for (int q = __ldg(I.df_thr_off + m0.z + i); q < q1; ++q) {
+        int4 rec = __ldg(I.df_rec + m0.x + q);       // slots of the block's touched list
+        rec.x = __ldg(I.df_touched + m0.y + rec.x);
+        if (rec.y >= 0) rec.y = __ldg(I.df_touched + m0.y + rec.y);
+        apply_event<NA>(a, X, r, rec, applied, clamped, skipped);
+      }
+    }
+  }
+  applied = __reduce_add_sync(0xffffffffu, applied);
+  clamped = __reduce_add_sync(0xffffffffu, clamped);
+  skipped = __reduce_add_sync(0xffffffffu, skipped);
+  if ((threadIdx.x & 31) == 0) {
+    unsigned long long* c = a.ctr + (size_t)r * 4;
+    if (applied) atomicAdd(c + 1, (unsigned long long)applied);
+    if (clamped) atomicAdd(c + 2, (unsigned long long)clamped);
+    if (skipped) atomicAdd(c + 3, (unsigned long long)skipped);
+  }
+}
+
+template <bool LISTS>
+__device__ __forceinline__ void dispatch_events(const BatchInst& I, int r, int day, int part, unsigned char* smem,
+                                                int smem_cap) {
   if (!I.has_events) return;
   const int dl0 = __ldg(I.evg.day_lvl + day), dl1 = __ldg(I.evg.day_lvl + day + 1);
   if (dl1 <= dl0) return;
+  if (LISTS && I.by_lists && __ldg(&I.day_df[day].y) > 0) {
+    if (I.na == 1) events_by_lists<1>(I, r, day, part); else events_by_lists<3>(I, r, day, part);
+    return;
+  }
+  if (part > 0) return;
   const int need = __ldg(I.day_smem + day);
   if (need > 0 && need <= smem_cap) {
     EvSmemArgs a = I.evs;
@@ -125,9 +170,10 @@ __device__ __forceinline__ void dispatch_events(const BatchInst& I, int r, int d
   }
 }
 
-// THREADS threads a block, MINB blocks an SM (the register budget), and whether
-// any instance computes the score (its stochastic step is compiled in only then).
-template <int THREADS, int MINB, bool SCORE_ANY>
+// THREADS threads a block, MINB blocks an SM (the register budget), whether any
+// instance computes the score and whether any takes its events by lists (either step is
+// compiled in only then: the lists' registers cost the batched national run 8 %).
+template <int THREADS, int MINB, bool SCORE_ANY, bool LISTS>
 __global__ void __launch_bounds__(THREADS, MINB) k_batch(BatchCtl c) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_item;
@@ -150,7 +196,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batch(BatchCtl c) {
       const long long local = t - c.step_off[s];
       const int act = c.active[s];
       const long long nA = c.cumA[act];
-      int k, r, chunk = 0;
+      int k, r, chunk = 0;                            // chunk: of the stochastic step, or part of the events
       const bool is_ssa = local < nA;
       if (is_ssa) {
         k = upper_index_from(c.cumA, act, (hs == s && hkind == 0) ? hk : 0, local);
@@ -160,23 +206,25 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batch(BatchCtl c) {
         chunk = (int)(w - (long long)r * I0.bpr);
       } else {
         k = upper_index_from(c.cumB, act, (hs == s && hkind == 1) ? hk : 0, local - nA);
-        r = (int)(local - nA - c.cumB[k]);
+        const long long w = local - nA - c.cumB[k];
+        const int parts = c.inst[k].ev_parts;
+        r = (int)(w / parts);
+        chunk = (int)(w - (long long)r * parts);
       }
       const BatchInst& I = c.inst[k];
       const int day = I.day0 + s;
-      if (threadIdx.x == 0) s_ok = is_ssa ? wait_at_least(I.ev_done + r, (unsigned)day, c)
+      if (threadIdx.x == 0) s_ok = is_ssa ? wait_at_least(I.ev_done + r, 1u + (unsigned)(s * I.ev_parts), c)
                                           : wait_at_least(I.ssa_done + r, (unsigned)((s + 1) * I.bpr), c);
       __syncthreads();
       if (s_ok) {
         if (is_ssa) dispatch_chunk<SCORE_ANY>(I, r, chunk, day, s > 0, 0);
-        else dispatch_events(I, r, day, smem, c.smem_cap);
+        else dispatch_events<LISTS>(I, r, day, chunk, smem, c.smem_cap);
       }
       __syncthreads();
       if (threadIdx.x == 0) { s_hs = s; s_hk = k; s_hkind = is_ssa ? 0 : 1; }   // read after the next barrier
       if (threadIdx.x == 0 && s_ok) {
         __threadfence();
-        if (is_ssa) atomicAdd(I.ssa_done + r, 1u);
-        else atomicMax(I.ev_done + r, (unsigned)(day + 1));
+        atomicAdd((is_ssa ? I.ssa_done : I.ev_done) + r, 1u);
       }
     } else {
       const long long local = t - c.total_main;
@@ -185,7 +233,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batch(BatchCtl c) {
       const long long w = local - c.cumF[k];
       const int r = (int)(w / I.tbpr), chunk = (int)(w - (long long)r * I.tbpr);
       const int last = I.day0 + I.ndays - 1;
-      if (threadIdx.x == 0) s_ok = wait_at_least(I.ev_done + r, (unsigned)(last + 1), c);
+      if (threadIdx.x == 0) s_ok = wait_at_least(I.ev_done + r, 1u + (unsigned)(I.ndays * I.ev_parts), c);
       __syncthreads();
       if (s_ok) dispatch_chunk<SCORE_ANY>(I, r, chunk, last, 1, 1);
     }
@@ -195,11 +243,17 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batch(BatchCtl c) {
 
 }  // namespace
 
-// The kernel of one block shape, with or without the score step compiled in; each
-// shape is instantiated in a translation unit of its own (batch_shape_*.cu).
+// The kernel of one block shape with the score step compiled in or not, and with the list
+// events; each is instantiated in a translation unit of its own (batch_shape_*.cu,
+// batch_lists_*.cu).
 template <int THREADS, int MINB>
-BatchKernel batch_kernel_of(bool score_any) {
-  return score_any ? (BatchKernel)k_batch<THREADS, MINB, true> : (BatchKernel)k_batch<THREADS, MINB, false>;
+BatchKernel batch_kernel_of(BatchForm f) {
+  return f == BatchForm::kScore ? (BatchKernel)k_batch<THREADS, MINB, true, false>
+                                : (BatchKernel)k_batch<THREADS, MINB, false, false>;
+}
+template <int THREADS, int MINB>
+BatchKernel batch_lists_of() {
+  return (BatchKernel)k_batch<THREADS, MINB, false, true>;
 }
 
 }  // namespace episim

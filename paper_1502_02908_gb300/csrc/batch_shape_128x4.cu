@@ -3,6 +3,6 @@
 
 namespace episim {
 
-BatchKernel batch_kernel_128x4(bool score_any) { return batch_kernel_of<128, 4>(score_any); }
+BatchKernel batch_kernel_128x4(BatchForm f) { return batch_kernel_of<128, 4>(f); }
 
 }  // namespace episim

@@ -3,6 +3,6 @@
 
 namespace episim {
 
-BatchKernel batch_kernel_256x1(bool score_any) { return batch_kernel_of<256, 1>(score_any); }
+BatchKernel batch_kernel_256x1(BatchForm f) { return batch_kernel_of<256, 1>(f); }
 
 }  // namespace episim

@@ -3,6 +3,6 @@
 
 namespace episim {
 
-BatchKernel batch_kernel_256x2(bool score_any) { return batch_kernel_of<256, 2>(score_any); }
+BatchKernel batch_kernel_256x2(BatchForm f) { return batch_kernel_of<256, 2>(f); }
 
 }  // namespace episim

@@ -133,6 +133,8 @@ struct sim_handle {
   int32_t* d_thr_id = nullptr;
   int32_t event_variant = 0;         // 0 auto, 1 global only, 2 levels (no owner-computes)
   int32_t* d_day_smem = nullptr;     // device copy for the persistent batch kernel
+  int2* d_day_df = nullptr;          // [max_days] its owner-list blocks of each day (BatchInst::day_df)
+  int32_t most_lists = 0;            // most of them on a day (0: no day's lists suit)
   std::vector<int64_t> sched_order;  // position in the day-stable order, execution order
   std::vector<int32_t> sched_level;
   std::vector<int32_t> day_lvl;      // [max_days + 1]
@@ -211,6 +213,9 @@ void free_events(sim_handle* h) {
   h->ev_first.clear();
   cudaFree(h->d_rec); cudaFree(h->d_lvl_start); cudaFree(h->d_day_lvl);
   cudaFree(h->d_rec_slot); cudaFree(h->d_touched); cudaFree(h->d_day_touch); cudaFree(h->d_day_smem);
+  cudaFree(h->d_day_df);
+  h->d_day_df = nullptr;
+  h->most_lists = 0;
   cudaFree(h->d_rec_df); cudaFree(h->d_wait_df); cudaFree(h->d_thr_off); cudaFree(h->d_touched_df);
   cudaFree(h->d_blk_meta); cudaFree(h->d_thr_id);
   h->d_rec_df = nullptr; h->d_wait_df = nullptr; h->d_thr_off = nullptr; h->d_touched_df = nullptr;
@@ -1351,7 +1356,24 @@ sim_status sim_load_events(sim_handle* h, int64_t n, const int32_t* day, const i
     h->day_smem[(size_t)d] = (b <= kEventsSmemLimit && !h->force_global_events) ? (int32_t)b : 0;
   }
   {
-    cudaError_t e2 = dalloc(&h->d_day_smem, (size_t)T);
+    // days whose owner lists the persistent kernel's lanes can take: every component owned
+    // whole, no list of more than kBatchEvLongest events, blocks enough to fill lanes
+    std::vector<int2> day_df((size_t)T, make_int2(0, 0));
+    for (int32_t d = 0; d < T; ++d) {
+      const int32_t b0 = S.day_blk[(size_t)d], b1 = S.day_blk[(size_t)d + 1];
+      bool suits = b1 - b0 >= 16;
+      for (int32_t b = b0; b < b1 && suits; ++b) {
+        const int4 m = S.blk_meta[(size_t)b];
+        suits = (m.w >> 16) != 0;
+        for (int32_t i = m.z; i + 1 < S.blk_meta[(size_t)b + 1].z && suits; ++i)
+          suits = S.thr_off[(size_t)i + 1] - S.thr_off[(size_t)i] <= kBatchEvLongest;
+      }
+      if (suits) day_df[(size_t)d] = make_int2(b0, b1 - b0);
+      h->most_lists = std::max(h->most_lists, day_df[(size_t)d].y);
+    }
+    cudaError_t e2 = dalloc(&h->d_day_df, (size_t)T);
+    if (e2 == cudaSuccess && T > 0) e2 = cudaMemcpy(h->d_day_df, day_df.data(), (size_t)T * sizeof(int2), cudaMemcpyHostToDevice);
+    if (e2 == cudaSuccess) e2 = dalloc(&h->d_day_smem, (size_t)T);
     if (e2 == cudaSuccess && T > 0) e2 = cudaMemcpy(h->d_day_smem, h->day_smem.data(), (size_t)T * 4, cudaMemcpyHostToDevice);
     if (e2 != cudaSuccess) { free_events(h); return cuda_fail(h, e2, "event upload"); }
   }
@@ -2208,12 +2230,22 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
   std::vector<long long> cumA(ni + 1, 0), cumB(ni + 1, 0), cumF(ni + 1, 0);
   long long n_counters = 0;
   int smem_cap = 0;
-  const BatchShape shape = g_batch_shape;
+  // The default shape gives way to one block an SM, with twice the registers a thread and
+  // fewer blocks polling, for runs whose per-thread nodes would not fill its blocks (32
+  // uneven instances: 54 ms a run against 73).
+  BatchShape shape = g_batch_shape;
+  {
+    long long nodes = 0;
+    for (int k = 0; k < ni; ++k) nodes += (long long)hs[idx[k]]->cfg.n_replicates * ((hs[idx[k]]->cfg.n_nodes + 255) / 256);
+    if (shape == BatchShape::k256x2 && nodes <= 2LL * hs[idx[0]]->sm_count) shape = BatchShape::k256x1;
+  }
   const int threads = batch_threads(shape);
   // two blocks an SM share its 228 KB of shared memory; a day whose staged event
   // step needs more takes the global-memory variant
   const int smem_limit = batch_min_blocks(shape) > 1 ? (int)(kBatchSmemSM / batch_min_blocks(shape)) : (int)kEventsSmemLimit;
-  bool score_any = false;
+  BatchForm form = BatchForm::kPlain;
+  for (int k = 0; k < ni; ++k)
+    if (hs[idx[k]]->cfg.flags & SIM_FLAG_SCORE) form = BatchForm::kScore;
   const int wpb = threads / 32;
   // the instances' automatic warp herds were chosen for each alone: together they keep
   // them while every unit still has a resident warp (chain_threshold otherwise)
@@ -2250,11 +2282,18 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
     I.n_thread = n_thread;
     I.bpr = I.ssa.warp_blocks + (n_thread + threads * subs - 1) / (threads * subs);
     I.tbpr = (h->cfg.n_nodes + threads - 1) / threads;
-    score_any = score_any || I.score;
     I.day0 = h->day;
     I.ndays = nd(idx[k]);
     I.has_events = h->events_loaded ? 1 : 0;
     I.day_smem = h->d_day_smem;
+    I.df_rec = h->d_rec_df; I.df_thr_off = h->d_thr_off; I.df_touched = h->d_touched_df; I.df_meta = h->d_blk_meta;
+    I.day_df = h->d_day_df;
+    I.ev_parts = 1;
+    if (h->events_loaded && h->event_variant == 0 && h->most_lists > 0 && form != BatchForm::kScore && shape != BatchShape::k128x4) {
+      form = BatchForm::kLists;
+      I.by_lists = 1;
+      I.ev_parts = std::min(16, (h->most_lists * kBatchEvLanes + threads - 1) / threads);
+    }
     EvArgs& ev = I.evg;
     ev.counts = h->d_counts; ev.rec = h->d_rec; ev.lvl_start = h->d_lvl_start; ev.day_lvl = h->d_day_lvl;
     ev.ctr = h->d_ctr; ev.err = h->d_err; ev.seed = h->cfg.seed; ev.rep_base = h->cfg.replicate_base;
@@ -2270,7 +2309,7 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
         if (h->day_smem[(size_t)d] <= smem_limit) smem_cap = std::max(smem_cap, h->day_smem[(size_t)d]);
     const long long R = h->cfg.n_replicates;
     cumA[k + 1] = cumA[k] + R * I.bpr;
-    cumB[k + 1] = cumB[k] + R;
+    cumB[k + 1] = cumB[k] + R * I.ev_parts;
     cumF[k + 1] = cumF[k] + R * I.tbpr;
     n_counters += 2 * R;
   }
@@ -2309,8 +2348,8 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
       inst[k].ssa_done = c + o;
       for (int r = 0; r < R; ++r) init[o++] = 0;
       inst[k].ev_done = c + o;
-      for (int r = 0; r < R; ++r) init[o++] = (unsigned)inst[k].day0;
-      if (g_batch_stall && k == 0) init[o - R] = 0;   // replicate 0 waits for a day that never comes
+      for (int r = 0; r < R; ++r) init[o++] = 1;
+      if (g_batch_stall && k == 0) init[o - R] = 0;   // replicate 0 waits for events that never come
     }
     cudaError_t e = cudaMemcpyAsync(d_ctr, init.data(), init.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_inst, inst.data(), bytes_inst, cudaMemcpyHostToDevice, st);
@@ -2332,13 +2371,13 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
   c.n_inst = ni; c.n_steps = S;
   c.smem_cap = smem_cap;
   int per_sm = 0, dev = 0, sms = 0;
-  cudaError_t e = batch_occupancy(shape, score_any, smem_cap, &per_sm);
+  cudaError_t e = batch_occupancy(shape, form, smem_cap, &per_sm);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
   const long long want = (long long)sms * per_sm;
   const int grid = (int)std::max(1LL, std::min(want, c.total));
-  if (e == cudaSuccess) e = launch_batch(c, shape, score_any, grid, st);
+  if (e == cudaSuccess) e = launch_batch(c, shape, form, grid, st);
   int berr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&berr, d_err, 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
