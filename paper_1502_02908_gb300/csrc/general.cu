@@ -409,7 +409,9 @@ __device__ __forceinline__ int32_t gen_thread_node_day(const GenSsaArgs& a, cons
 // lists and no read-modify-write chains), and takes the rates, sums and choice of the
 // thread method: about 150 instructions and 450 cycles for six transitions, against
 // 2,800 cycles for a pass over transitions, counts and sums in shared memory one by
-// one.  EXACT (SEG = 32): the clock of each lane's draw in binary64 (tau of its state,
+// one.  Where every change is -1, 0 or 1 and at most 16 rows move, the state comes from
+// byte sums instead: a lane's choice as one byte (change + 1) a row, four rows a word,
+// summed over the lanes below in log2(SEG) shuffles a word (at most 64 a byte).  EXACT (SEG = 32): the clock of each lane's draw in binary64 (tau of its state,
 // summed exactly in Q62; a decision is certain outside (k + 2) 2^-52), for node-days
 // whose binary32 clock was too close to call.  Otherwise tau~ = E~ / a0~ (neglog_f32:
 // 16u) goes through a binary32 scan of the round, whose start is a binary32 pair:
@@ -420,8 +422,8 @@ __device__ __forceinline__ int32_t gen_thread_node_day(const GenSsaArgs& a, cons
 // to call, or a state out of bounds): base then no longer holds the day's start.
 template <int L, int SEG, bool EXACT>
 __device__ __forceinline__ int32_t gen_draws_node_day(const GenSsaArgs& a, const GenModelDev& m, const GenRepParams& p,
-                                                      const float* S, const float (&kyf)[L], float* xf, float* base,
-                                                      const double* y, uint32_t v, uint32_t rep, uint32_t k0,
+                                                      const float* S, const uint32_t* pk, const float (&kyf)[L],
+                                                      float* xf, float* base, const double* y, uint32_t v, uint32_t rep, uint32_t k0,
                                                       uint32_t k1, bool live, float margin) {
   const unsigned full = 0xffffffffu;
   const unsigned seg = SEG == 32 ? full : ((1u << (SEG & 31)) - 1u);
@@ -443,19 +445,45 @@ __device__ __forceinline__ int32_t gen_draws_node_day(const GenSsaArgs& a, const
     float sc = 0.0f;
     bool bad = false, valid = false, sure = false;
     for (int it = 0; it <= SEG; ++it) {
-      float cnt[L];
-#pragma unroll
-      for (int n = 0; n < L; ++n)
-        cnt[n] = n < nt ? __int2float_rn(__popc(__ballot_sync(full, choice == n) & below)) : 0.0f;
       float least = 0.0f, most = 0.0f;
-      for (int r = 0; r < rows; ++r) {
-        float x = base[r];
-        const float* Sr = S + r * L;
+      if (a.pk_words > 0) {
+        const float back = __int2float_rn(sl);
 #pragma unroll
-        for (int n = 0; n < L; ++n) x = __fmaf_rn(Sr[n], cnt[n], x);
-        least = fminf(least, x);
-        most = fmaxf(most, x);
-        xf[r * kGenThreads] = x;
+        for (int q = 0; q < 4; ++q) {
+          if (q >= a.pk_words) break;
+          const uint32_t own = choice >= 0 ? pk[choice * a.pk_words + q] : 0x01010101u;
+          uint32_t sum = own;
+#pragma unroll
+          for (int o = 1; o < SEG; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(full, sum, o, SEG);
+            if (sl >= o) sum += t;
+          }
+          sum -= own;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = 4 * q + i;
+            if (r < rows) {
+              const float x = __fadd_rn(base[r], __fsub_rn(__uint2float_rn((sum >> (8 * i)) & 0xffu), back));
+              least = fminf(least, x);
+              most = fmaxf(most, x);
+              xf[r * kGenThreads] = x;
+            }
+          }
+        }
+      } else {
+        float cnt[L];
+#pragma unroll
+        for (int n = 0; n < L; ++n)
+          cnt[n] = n < nt ? __int2float_rn(__popc(__ballot_sync(full, choice == n) & below)) : 0.0f;
+        for (int r = 0; r < rows; ++r) {
+          float x = base[r];
+          const float* Sr = S + r * L;
+#pragma unroll
+          for (int n = 0; n < L; ++n) x = __fmaf_rn(Sr[n], cnt[n], x);
+          least = fminf(least, x);
+          most = fmaxf(most, x);
+          xf[r * kGenThreads] = x;
+        }
       }
       bad = least < 0.0f || most >= kGenBigCount;
       float P[L];
@@ -559,10 +587,11 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
   GenModelDev& m = *reinterpret_cast<GenModelDev*>(smem4);
   char* sp = reinterpret_cast<char*>(smem4) + sizeof(GenModelDev);
   copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
-  // the change tables: [dyn_rows][L], then the thread method's [nt] and longer lists
+  // the change tables: [dyn_rows][L], the thread method's [nt], bytes [nt][pk_words], longer lists
   float* S = reinterpret_cast<float*>(sp);
   int4* chg = reinterpret_cast<int4*>(S + a.dyn_rows * L);
-  int2* more = reinterpret_cast<int2*>(chg + a.nt);
+  const uint32_t* pk = reinterpret_cast<const uint32_t*>(chg + a.nt);
+  const int2* more = reinterpret_cast<const int2*>(pk + a.nt * a.pk_words + (a.nt * a.pk_words & 1));
   copy16(S, a.tab, a.tab16);
   sp += (size_t)a.tab16 * 16;
   double* ctau = reinterpret_cast<double*>(sp);                 // [threads]: per lane
@@ -694,11 +723,11 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
     } else if (role == 1) {
       const unsigned oks = __ballot_sync(full, ok);
       const bool live = has && ((oks >> sb) & ((1u << kGenSeg) - 1u)) == (1u << kGenSeg) - 1u;
-      const int32_t g = gen_draws_node_day<L, kGenSeg, false>(a, m, p, S, kyf, xf, base, y, (uint32_t)v, rep, k0, k1,
+      const int32_t g = gen_draws_node_day<L, kGenSeg, false>(a, m, p, S, pk, kyf, xf, base, y, (uint32_t)v, rep, k0, k1,
                                                               live, a.margin_f);
       if (live) f = g;
     } else if (__all_sync(full, ok)) {
-      f = gen_draws_node_day<L, 32, false>(a, m, p, S, kyf, xf, base, y, (uint32_t)v, rep, k0, k1, true, a.margin_f);
+      f = gen_draws_node_day<L, 32, false>(a, m, p, S, pk, kyf, xf, base, y, (uint32_t)v, rep, k0, k1, true, a.margin_f);
     }
     if (role != 2 && has && f >= 0)
       for (int c = sl; c < nc; c += width) {
@@ -737,7 +766,7 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
         if (lane < nc) bl[lane] = __int2float_rn(rl[lane]);
         if (lane == 0) { bl[nc + a.npop] = 1.0f; bl[nc + a.npop + 1] = 0.0f; }
         __syncwarp();
-        n = gen_draws_node_day<L, 32, true>(a, m, p, S, kl, xf, bl, yl, (uint32_t)vl, rep, k0, k1, true, 0.0f);
+        n = gen_draws_node_day<L, 32, true>(a, m, p, S, pk, kl, xf, bl, yl, (uint32_t)vl, rep, k0, k1, true, 0.0f);
         if (n >= 0 && lane < nc) rl[lane] = (int32_t)bl[lane];
         __syncwarp();
       }

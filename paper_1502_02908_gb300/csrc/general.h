@@ -55,10 +55,11 @@ struct GenSsaArgs {
   float margin_f;               // the same as binary32
   // Change tables, back to back (tab16 16-byte words): [dyn_rows][L] floats, what transition
   // n adds to row r; the thread method's [nt] {row0 | row1 << 16, change0 | change1 << 16,
-  // first, end of further changes} and those {row, change} pairs (rows in elements of a
-  // thread's column).
+  // first, end of further changes}; [nt][pk_words] words of four rows' change + 1 a byte;
+  // the further {row, change} pairs (rows in elements of a thread's column).
   const float4* tab;
   int32_t tab16;
+  int32_t pk_words;             // words of the byte table (0: a change beyond -1..1, or too many rows)
   int32_t nt, L;                // transitions; the power of two the kernel is unrolled for
   int32_t resident_blocks;      // blocks the device holds at once
   int32_t xrows;                // rows of a thread's column: counts, populations, ones, scratch

@@ -204,10 +204,19 @@ void build_tables(const GenModelDev& md, const int32_t* stoich, GenSsaArgs* s, s
     more.insert(more.end(), ch.begin() + 2, ch.end());
   }
   const size_t dense16 = dense.size() / 4;                      // L is a multiple of 4
-  tab.assign(dense16 + first.size() + (more.size() + 1) / 2 + 1, make_float4(0.f, 0.f, 0.f, 0.f));
+  bool unit = s->dyn_rows <= 16;
+  for (float d : dense) unit = unit && d >= -1.f && d <= 1.f;
+  s->pk_words = unit ? (s->dyn_rows + 3) / 4 : 0;
+  std::vector<uint32_t> bytes((size_t)nt * s->pk_words + ((size_t)nt * s->pk_words & 1), 0x01010101u);
+  for (int n = 0; unit && n < nt; ++n)
+    for (int r = 0; r < s->dyn_rows; ++r)
+      bytes[(size_t)n * s->pk_words + r / 4] += (uint32_t)(int)dense[(size_t)r * L + n] << (8 * (r % 4));
+  tab.assign(dense16 + first.size() + (bytes.size() / 2 + more.size() + 1) / 2 + 1, make_float4(0.f, 0.f, 0.f, 0.f));
   std::memcpy(tab.data(), dense.data(), dense.size() * sizeof(float));
   if (nt) std::memcpy(&tab[dense16], first.data(), first.size() * sizeof(int4));
-  if (!more.empty()) std::memcpy(&tab[dense16 + first.size()], more.data(), more.size() * sizeof(int2));
+  char* rest = reinterpret_cast<char*>(&tab[dense16 + first.size()]);
+  if (!bytes.empty()) std::memcpy(rest, bytes.data(), bytes.size() * 4);
+  if (!more.empty()) std::memcpy(rest + bytes.size() * 4, more.data(), more.size() * sizeof(int2));
   s->tab16 = (int32_t)tab.size();
 }
 
