@@ -586,6 +586,7 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
   extern __shared__ int4 smem4[];
   GenModelDev& m = *reinterpret_cast<GenModelDev*>(smem4);
   char* sp = reinterpret_cast<char*>(smem4) + sizeof(GenModelDev);
+  grid_dependents_launch();
   copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
   // the change tables: [dyn_rows][L], the thread method's [nt], bytes [nt][pk_words], longer lists
   float* S = reinterpret_cast<float*>(sp);
@@ -623,6 +624,7 @@ __global__ void __launch_bounds__(kGenThreads, 4) k_gen_ssa(GenSsaArgs a) {
   const bool midpoint = m.y_source == kGenYMidpoint, pre_event = m.y_source == kGenYPreEvent;
   float* xf = xfs + threadIdx.x;
   int32_t* xi = reinterpret_cast<int32_t*>(xf);
+  grid_dependency_wait();                                       // counts and variables of the previous step
   for (uint32_t u = (uint32_t)warp * gridDim.x + blockIdx.x; u < units; u += T) {
     // role 0: a warp node; 1: four nodes on segments; 2: 32 nodes
     const int role = u < uw ? 0 : (u < uw + ug ? 1 : 2);
@@ -794,6 +796,8 @@ __global__ void __maxnreg__(128) k_gen_ssa_exact(GenSsaArgs a) {
   extern __shared__ int4 smem4[];
   GenModelDev& m = *reinterpret_cast<GenModelDev*>(smem4);
   char* sp = reinterpret_cast<char*>(smem4) + sizeof(GenModelDev);
+  grid_dependents_launch();
+  grid_dependency_wait();
   GenRepParams& p = *reinterpret_cast<GenRepParams*>(sp);
   sp += sizeof(GenRepParams);
   double* ctau = reinterpret_cast<double*>(sp);                 // [threads]: per lane
@@ -917,6 +921,7 @@ __global__ void __maxnreg__(128) k_gen_ssa_exact(GenSsaArgs a) {
 __global__ void __launch_bounds__(kGenThreads) k_gen_events(GenEvArgs a) {
   __shared__ GenModelDev m;
   __shared__ int32_t cache[kGenMaxComp * kGenThreads];
+  grid_dependents_launch();
   copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
   __syncthreads();
   const int r = blockIdx.y, nc = m.nc, N = a.N;
@@ -934,6 +939,7 @@ __global__ void __launch_bounds__(kGenThreads) k_gen_events(GenEvArgs a) {
     int e_next = 0;
     int4 rec_next = make_int4(0, 0, 0, 0);
     if (pi < p1) { e_next = __ldg(a.comp_ev + pi); rec_next = __ldg(a.rec + pi); }
+    grid_dependency_wait();                          // the stochastic step's counts
     for (; pi < p1; ++pi) {
       const int e = e_next;
       const int4 rec = rec_next;
@@ -993,6 +999,7 @@ __global__ void __launch_bounds__(kGenThreads) k_gen_events(GenEvArgs a) {
     if (cur >= 0)
       for (int c = 0; c < nc; ++c) X[(size_t)c * N + cur] = cc[c * S];
   }
+  grid_dependency_wait();                            // threads without a component too
   const uint32_t sa = __reduce_add_sync(0xffffffffu, applied);
   const uint32_t sc = __reduce_add_sync(0xffffffffu, clamped);
   const uint32_t ss = __reduce_add_sync(0xffffffffu, skipped);
@@ -1011,9 +1018,11 @@ __global__ void __launch_bounds__(kGenThreads) k_gen_cont(GenContArgs a) {
   __shared__ GenModelDev m;
   __shared__ GenRepParams p;
   const int r = blockIdx.y;
+  grid_dependents_launch();
   copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
   copy16(&p, a.params + r, (int)(sizeof(GenRepParams) / 16));
   __syncthreads();
+  grid_dependency_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x, N = a.N, nc = m.nc, ny = m.ny;
   if (v >= N) return;
   const int32_t* X = a.counts + (size_t)r * nc * N + v;
@@ -1080,17 +1089,15 @@ cudaError_t launch_gen_ssa(GenSsaArgs a, int nt, int nc, cudaStream_t st) {
     a.group_blocks = (a.n_mid + per_block - 1) / per_block;
     const int rest = a.N - a.n_big - a.n_mid;
     const dim3 grid((unsigned)(a.warp_blocks + a.group_blocks + (rest + kGenThreads - 1) / kGenThreads), (unsigned)a.R);
-    k_gen_ssa_exact<<<grid, kGenThreads, gen_ssa_smem_bytes(nc, nt), st>>>(a);
-    return cudaGetLastError();
+    return launch_maybe_pdl(k_gen_ssa_exact, grid, dim3(kGenThreads), gen_ssa_smem_bytes(nc, nt), st, true, a);
   }
   // resident grid, fewer blocks when the units do not fill it (one unit a warp)
   const int64_t per = 32 / kGenSeg;
   const int64_t units =
       (int64_t)a.R * (a.n_big + ((int64_t)a.n_mid + per - 1) / per + ((int64_t)a.N - a.n_big - a.n_mid + 31) / 32);
   const int64_t grid = std::min<int64_t>(a.resident_blocks, (units + kGenWarps - 1) / kGenWarps);
-  gen_ssa_kernel(a.L)<<<(unsigned)std::max<int64_t>(grid, 1), kGenThreads, 
-                               gen_f32_smem_bytes(nc, nt, a.L, a.tab16, a.xrows), st>>>(a);
-  return cudaGetLastError();
+  return launch_maybe_pdl(gen_ssa_kernel(a.L), dim3((unsigned)std::max<int64_t>(grid, 1)), dim3(kGenThreads),
+                          gen_f32_smem_bytes(nc, nt, a.L, a.tab16, a.xrows), st, true, a);
 }
 
 cudaError_t launch_gen_events(const GenEvArgs& a, cudaStream_t st) {
@@ -1098,14 +1105,12 @@ cudaError_t launch_gen_events(const GenEvArgs& a, cudaStream_t st) {
   // a warp per component up to kGenEventWarps warps, then up to 32 per warp
   const int warps = std::max((a.ncomp + 31) / 32, std::min(a.ncomp, kGenEventWarps));
   const dim3 grid((unsigned)((warps + kGenWarps - 1) / kGenWarps), (unsigned)a.R);
-  k_gen_events<<<grid, kGenThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_maybe_pdl(k_gen_events, grid, dim3(kGenThreads), 0, st, true, a);
 }
 
 cudaError_t launch_gen_cont(const GenContArgs& a, cudaStream_t st) {
   const dim3 grid((unsigned)((a.N + kGenThreads - 1) / kGenThreads), (unsigned)a.R);
-  k_gen_cont<<<grid, kGenThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_maybe_pdl(k_gen_cont, grid, dim3(kGenThreads), 0, st, true, a);
 }
 
 }  // namespace episim
