@@ -229,6 +229,7 @@ __device__ __forceinline__ uint32_t gen_seg_node_day(const GenModelDev& m, const
 constexpr int kGenSeg = 8;                          // lanes per node of the group method
 constexpr int kGenWarps = kGenThreads / 32;
 constexpr int kGenEventWarps = 8192;                // event step: a warp per component up to this many
+constexpr int kGenSmall = 4;                         // event step: compartments that stay in registers
 
 // ---------------------------------------------------------------------------
 // Binary32 methods.  With u = 2^-24, nt <= 32, every constant k_j y_q 0 or within
@@ -909,6 +910,43 @@ __global__ void __maxnreg__(128) k_gen_ssa_exact(GenSsaArgs a) {
   if (lane == 0 && tot) atomicAdd(a.ctr + (size_t)r * 4, (unsigned long long)tot);
 }
 
+// `take` of the animals counted by h (their sum, avail, above `take`), uniformly and one
+// at a time, from the event's word stream, whose first Philox block comes with the call
+// (w).  A draw is compared with the running sums of what is left, all at once; WIDE, for
+// a sum past 32 bits (entries alone can get there), walks the compartments instead.
+template <bool WIDE, int C>
+__device__ __forceinline__ void gen_take(const int32_t (&h)[C], int64_t avail, int take, uint4 w, uint32_t e,
+                                         uint32_t tag, uint32_t rep, uint32_t k0, uint32_t k1, int32_t (&took)[C]) {
+  uint32_t cum[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    cum[c] = (uint32_t)h[c] + (c && !WIDE ? cum[c > 0 ? c - 1 : 0] : 0u);
+  }
+  uint32_t wq = 0;
+  auto next = [&]() -> uint32_t {
+    const uint32_t s = wq & 3u;
+    if (s == 0u && wq) w = philox10(make_uint4(e, tag, wq >> 2, rep), k0, k1);
+    ++wq;
+    return s == 0 ? w.x : s == 1 ? w.y : s == 2 ? w.z : w.w;
+  };
+#pragma unroll 1
+  for (int t = 0; t < take; ++t) {
+    uint32_t slot = lemire((uint32_t)(avail - t), next);
+    bool open = true;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const bool hit = open && slot < cum[c];
+      if (WIDE) {
+        open = open && !hit;
+        slot -= open ? cum[c] : 0u;
+      }
+      cum[c] -= hit ? 1u : 0u;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) took[c] = h[c] - (int32_t)(cum[c] - (c && !WIDE ? cum[c > 0 ? c - 1 : 0] : 0u));
+}
+
 // One thread per component of the day's transfer graph: its events in input
 // order (no other thread touches its nodes this day).  Components (largest first)
 // are dealt lane-major over the grid's warps: component i runs on lane i / W of
@@ -1011,6 +1049,146 @@ __global__ void __launch_bounds__(kGenThreads) k_gen_events(GenEvArgs a) {
   }
 }
 
+// The event step for models of up to four compartments, dealt as in k_gen_events.  What
+// bounds it is one thread's chain of latencies, so nothing in it waits that need not:
+// the records come two events ahead, the next event's first Philox block and the counts
+// of the node it samples one ahead (the first of them before the stochastic step is
+// done); the counts of the node being sampled stay in registers with the running sums
+// that a draw is compared with all at once; transfers leave as reductions, which nobody
+// waits for.  A destination is never the node in the registers, and a node that the
+// current event adds to is not read ahead.  A launch of a SEIRS day (about 2,600
+// components): 9.6 -> 8.4 us; a year of it 13.9 -> 12.7 ms, 60 days of SIR with 2,000
+// nodes 0.92 -> 0.77 ms.  For more compartments the fixed work per event outgrows what
+// the row in shared memory costs on the long chains of a hub herd: six compartments,
+// 37,000 herds, a year: 11.2 -> 10.7 ms on some schedules, 13.4 -> 13.9 on those with
+// longer chains, so those keep k_gen_events.
+template <int C>
+__global__ void __launch_bounds__(kGenThreads) k_gen_events_small(GenEvArgs a) {
+  __shared__ GenModelDev m;
+  grid_dependents_launch();
+  copy16(&m, a.model, (int)(sizeof(GenModelDev) / 16));
+  __syncthreads();
+  const int r = blockIdx.y, nc = m.nc, N = a.N;
+  const int W = (int)gridDim.x * (int)(blockDim.x >> 5);
+  const int ci = (int)(threadIdx.x & 31) * W + (int)blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
+  uint32_t applied = 0, clamped = 0, skipped = 0;
+  if (ci < a.ncomp) {
+    int32_t* X = a.counts + (size_t)r * nc * N;
+    const uint32_t rep = (uint32_t)(a.rep_base + r);
+    uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
+    const uint32_t tag = (uint32_t)a.day | kEventTag;
+    auto load_row = [&](int v, int32_t (&x)[C]) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) x[c] = c < nc ? __ldcg(X + (size_t)c * N + v) : 0;
+    };
+    auto store_row = [&](int v, const int32_t (&x)[C]) {
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (c < nc) X[(size_t)c * N + v] = x[c];
+    };
+    int pi = a.comp_off[a.comp0 + ci];
+    const int p1 = a.comp_off[a.comp0 + ci + 1];
+    int4 rec = __ldg(a.rec + pi), rec1 = rec;        // a component has at least one event
+    int e = __ldg(a.comp_ev + pi), e1 = e;
+    if (pi + 1 < p1) { rec1 = __ldg(a.rec + pi + 1); e1 = __ldg(a.comp_ev + pi + 1); }
+    uint4 w = philox10(make_uint4((uint32_t)e, tag, 0u, rep), k0, k1);
+    grid_dependency_wait();                          // the stochastic step's counts
+    int32_t x[C];
+    load_row(rec.x, x);
+#pragma unroll 1
+    for (; pi < p1; ++pi) {
+      asm volatile("" : "+r"(k0), "+r"(k1));        // keep the ten round keys out of registers
+      int4 rec2 = rec1;
+      int e2 = e1;
+      if (pi + 2 < p1) { rec2 = __ldg(a.rec + pi + 2); e2 = __ldg(a.comp_ev + pi + 2); }
+      const int node = rec.x, dest = rec.y, n = rec.z;
+      const int kind = rec.w & 0xff, sel = (rec.w >> 8) & 0xff, sh = (rec.w >> 16) & 0xff;
+      const bool move = pi + 1 < p1 && rec1.x != node;
+      const bool ahead = move && !(kind == SIM_EXTERNAL && dest == rec1.x);
+      int32_t nx[C];
+      if (ahead) load_row(rec1.x, nx);
+      const uint4 w1 = philox10(make_uint4((uint32_t)e1, tag, 0u, rep), k0, k1);
+      const uint32_t mask = m.select[sel];
+      const int8_t* off = m.shift[sh];
+      if (kind == SIM_ENTER) {
+        const int c0 = __ffs(mask) - 1, to = c0 + off[c0];
+#pragma unroll
+        for (int c = 0; c < C; ++c) x[c] += c == to ? n : 0;
+        ++applied;
+      } else {
+        int32_t h[C], took[C];
+        long long avail = 0;
+        int kinds = 0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          h[c] = (mask >> c & 1u) ? x[c] : 0;
+          avail += h[c];
+          kinds += h[c] > 0 ? 1 : 0;
+        }
+        int take = n;
+        bool apply = true;
+        if ((long long)n > avail) {
+          if (a.underflow_error) {
+            ++skipped;
+            atomicOr(a.err, 1);
+            apply = false;
+          } else {
+            take = (int)avail;
+            ++clamped;
+          }
+        }
+        if (apply) {
+          // every animal, or animals of one compartment: whatever the draws
+          if (take == avail || kinds <= 1) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) took[c] = h[c] > take ? take : h[c];
+          } else if (avail >> 32) {
+            gen_take<true, C>(h, avail, take, w, (uint32_t)e, tag, rep, k0, k1, took);
+          } else {
+            gen_take<false, C>(h, avail, take, w, (uint32_t)e, tag, rep, k0, k1, took);
+          }
+#pragma unroll
+          for (int c = 0; c < C; ++c) x[c] -= took[c];
+          if (kind != SIM_EXIT) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+              if (!took[c]) continue;
+              const int to = c + off[c];
+              if (kind == SIM_EXTERNAL) {
+                atomicAdd(&X[(size_t)to * N + dest], took[c]);
+              } else {                               // never into the mask (checked at load)
+#pragma unroll
+                for (int k = 0; k < C; ++k) x[k] += k == to ? took[c] : 0;
+              }
+            }
+          }
+          ++applied;
+        }
+      }
+      if (move) {
+        store_row(node, x);
+        if (!ahead) load_row(rec1.x, nx);
+#pragma unroll
+        for (int c = 0; c < C; ++c) x[c] = nx[c];
+      } else if (pi + 1 >= p1) {
+        store_row(node, x);
+      }
+      rec = rec1; e = e1; w = w1;
+      rec1 = rec2; e1 = e2;
+    }
+  }
+  grid_dependency_wait();                            // threads without a component too
+  const uint32_t sa = __reduce_add_sync(0xffffffffu, applied);
+  const uint32_t sc = __reduce_add_sync(0xffffffffu, clamped);
+  const uint32_t ss = __reduce_add_sync(0xffffffffu, skipped);
+  if ((threadIdx.x & 31) == 0) {
+    unsigned long long* C4 = a.ctr + (size_t)r * 4;
+    if (sa) atomicAdd(C4 + 1, (unsigned long long)sa);
+    if (sc) atomicAdd(C4 + 2, (unsigned long long)sc);
+    if (ss) atomicAdd(C4 + 3, (unsigned long long)ss);
+  }
+}
+
 // Continuous update of a run's last day from the post-event counts, or the
 // midpoint with the sums the stochastic step saved (earlier days' updates run in
 // the next day's stochastic-step prologue).
@@ -1062,6 +1240,11 @@ GenSsaKernel gen_ssa_kernel(int L) {
   return L == 4 ? k_gen_ssa<4> : L == 8 ? k_gen_ssa<8> : L == 16 ? k_gen_ssa<16> : k_gen_ssa<32>;
 }
 
+using GenEventsKernel = void (*)(GenEvArgs);
+GenEventsKernel gen_events_kernel(int nc) {
+  return nc <= kGenSmall ? k_gen_events_small<kGenSmall> : k_gen_events;
+}
+
 }  // namespace
 
 // Transitions the kernel is unrolled for: the power of two that holds the model's.
@@ -1100,12 +1283,12 @@ cudaError_t launch_gen_ssa(GenSsaArgs a, int nt, int nc, cudaStream_t st) {
                           gen_f32_smem_bytes(nc, nt, a.L, a.tab16, a.xrows), st, true, a);
 }
 
-cudaError_t launch_gen_events(const GenEvArgs& a, cudaStream_t st) {
+cudaError_t launch_gen_events(const GenEvArgs& a, int nc, cudaStream_t st) {
   if (a.ncomp <= 0) return cudaSuccess;
   // a warp per component up to kGenEventWarps warps, then up to 32 per warp
   const int warps = std::max((a.ncomp + 31) / 32, std::min(a.ncomp, kGenEventWarps));
   const dim3 grid((unsigned)((warps + kGenWarps - 1) / kGenWarps), (unsigned)a.R);
-  return launch_maybe_pdl(k_gen_events, grid, dim3(kGenThreads), 0, st, true, a);
+  return launch_maybe_pdl(gen_events_kernel(nc), grid, dim3(kGenThreads), 0, st, true, a);
 }
 
 cudaError_t launch_gen_cont(const GenContArgs& a, cudaStream_t st) {

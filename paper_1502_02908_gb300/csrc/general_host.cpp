@@ -292,7 +292,7 @@ sim_status enqueue_days(gen_handle* h, int32_t d0, int32_t nd, cudaStream_t st) 
       e.comp0 = c0; e.ncomp = c1 - c0; e.model = h->d_model; e.ctr = h->d_ctr; e.err = h->d_err;
       e.seed = h->cfg.seed; e.rep_base = h->cfg.replicate_base; e.N = N; e.R = R; e.day = d;
       e.underflow_error = h->cfg.underflow_policy == SIM_UNDERFLOW_ERROR;
-      GCK(h, launch_gen_events(e, st), "event step launch");
+      GCK(h, launch_gen_events(e, h->nc, st), "event step launch");
     }
   }
   // the last day's continuous update (earlier days' run in the next day's prologue)
