@@ -153,16 +153,9 @@ __device__ __forceinline__ float small_int_to_f32(int32_t n) {  // exact for 0 <
   return __fsub_rn(__int_as_float(0x4B000000 | n), 8388608.0f);
 }
 
-// -1: a < b decisively, +1: a > b decisively, 0: too close to call in FP32.
-__device__ __forceinline__ int cmp_f32(float a, float b) {
-  const int ia = __float_as_int(a), ib = __float_as_int(b);
-  if (ia < 0x00800000 || ib < 0x00800000) return 0;  // zero or subnormal: exact path
-  const int d = ia - ib;
-  return d <= -64 ? -1 : (d >= 64 ? 1 : 0);
-}
-
 // ---------------------------------------------------------------------------
-// Speculative binary32 clock.  The specification's clock is the binary64 chain
+// Speculative binary32 clock, in the form of the eight-lane group method (the others
+// derive theirs at ssa_node_day_spec and ssa_warp_day_spec).  The specification's clock is the binary64 chain
 // t_{k+1} = fl(t_k + fl(E_k / a0_k)) and a day ends at the first k with
 // t_{k+1} >= 1.  Here tau~_k = E~_k / a0~_k in binary32 (E~ the binary32 -log of
 // the draw below, a0~ the binary32 propensity sum) is accumulated exactly in Q62
@@ -170,13 +163,13 @@ __device__ __forceinline__ int cmp_f32(float a, float b) {
 // binary32: 2u, product u, three sums u each), E~ within 16u of E, and the
 // division (__fdividef, 2 ulps) adds 4u, so tau~_k is within rho = 26u < 2^-19.2
 // of tau_k.  At a decision the Q62 sum is below 2.5, hence within 2.5 rho
-// (< 2^-17.9) plus k (2^-53 + 2^-62) of the binary64 chain for k < 2^24: a margin of 2^-17 makes
+// (< 2^-17.9) plus k (2^-53 + 2^-62) of the binary64 chain for k < 2^24: a margin of 2^-17 (the
+// narrowest one allowed) makes
 // "sum >= 1 + margin" a certain stop and "sum + margin < 1" a certain continue;
 // anything between is handed to the exact binary64 method.  The stochastic
 // choices are taken in binary32 only when decisive (below) and in binary64
 // otherwise, so the result is the specification's, bit for bit.
 constexpr uint64_t kQ62One = 1ull << 62;
-constexpr uint64_t kClockMargin = kQ62One >> 17;   // largest allowed margin exponent: 17
 constexpr uint32_t kSpecMaxSteps = 1u << 24;
 
 // binary32 of m 2^-53 for 1 <= m < 2^53, rounded to nearest (ties away): within u.
