@@ -1255,13 +1255,25 @@ int gen_unroll(int nt) {
   return L;
 }
 
+// The limit belongs to the kernel, which every handle of its unrolled size shares: it is
+// raised to what the device allows, never to one handle's own need, so that no handle
+// lowers it for another.
+static cudaError_t allow_smem(const void* k) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+  return e;
+}
+
 cudaError_t gen_ssa_prepare(int nc, int nt, int L, int tab16, int xrows, int* blocks_per_sm) {
   const GenSsaKernel k = gen_ssa_kernel(L);
-  const size_t smem = gen_f32_smem_bytes(nc, nt, L, tab16, xrows), exact = gen_ssa_smem_bytes(nc, nt);
-  cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024) e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && exact > 48 * 1024)
-    e = cudaFuncSetAttribute((const void*)k_gen_ssa_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact);
+  const size_t smem = gen_f32_smem_bytes(nc, nt, L, tab16, xrows);
+  cudaError_t e = allow_smem((const void*)k);
+  if (e == cudaSuccess) e = allow_smem((const void*)k_gen_ssa_exact);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)k, kGenThreads, smem);
   return e;
 }

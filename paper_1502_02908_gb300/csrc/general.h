@@ -92,7 +92,8 @@ struct GenContArgs {
 };
 
 int gen_unroll(int nt);
-// Shared-memory limits of the stochastic-step kernels and the blocks an SM holds (once per handle).
+// Raises the shared-memory limits of the stochastic-step kernels to the device's; the blocks an
+// SM holds of this model's.
 cudaError_t gen_ssa_prepare(int nc, int nt, int L, int tab16, int xrows, int* blocks_per_sm);
 cudaError_t launch_gen_ssa(GenSsaArgs a, int nt, int nc, cudaStream_t st);
 cudaError_t launch_gen_events(const GenEvArgs& a, int nc, cudaStream_t st);
