@@ -325,8 +325,10 @@ int32_t sim_warp_nodes(const sim_handle* h);
  *     disables it.
  *   SIM_OPT_CLOCK_MARGIN: k in [0, 17].  The stochastic step (outside score
  *     mode) first runs each node-day with a binary32 clock, whose distance to the
- *     binary64 clock of Eq. (numstep3) is bounded below 2^-17 of a day; a stop/continue decision within 2^-k of the day's end
- *     reruns the node-day with the exact binary64 arithmetic.  k = 17 (default)
+ *     binary64 clock of Eq. (numstep3) is bounded below 2^-17 of a day plus a term
+ *     in the reciprocals of the propensity sums; a stop/continue decision within
+ *     2^-k and that term of the day's end reruns the node-day with the exact
+ *     binary64 arithmetic.  k = 17 (default)
  *     is the tightest safe margin; smaller k only reruns more node-days; 0 runs
  *     every node-day exactly.  Values outside [0, 17]: SIM_E_INVALID_ARG.
  *   SIM_OPT_OVERLAP: 1 (default) launches the day's stochastic-step and event

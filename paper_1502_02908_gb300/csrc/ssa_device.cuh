@@ -587,9 +587,12 @@ __device__ __forceinline__ int32_t ssa_node_day_spec(const DevParams& p, uint64_
 //
 // In a round's passes, a binary32 clock: tau~ = E~ / a0~ (E~ within u and 2^-38, a0~
 // 6u, the reciprocal 2u, the product u) scanned over the round (5u) and added to the
-// round's start (u): within 20u plus 2^-38 sum(1 / a0~) of the binary64 chain, against
-// a margin of 2^-17 = 128u.  The first draw that is not a certain continue ends the
-// day when it is a certain stop.
+// round's start (u): within 20u t plus 2^-38 sum(1 / a0~) of the binary64 chain, against
+// a margin of 2^-17 = 128u.  Draws that are taken as continues have a0~ >= 2^-12, so the
+// sum over them stays below 2^-18 (rsum below, and 2^-21 for the round's own).  The
+// first draw that is not a certain continue ends the day when it is a certain stop:
+// d >= margin + 2^-37 / a0~, since its own a0~ may be as small as 2^-100, where E~'s
+// absolute error is many days (its tau~ is not clipped: 2^106 at most).
 //
 // Between rounds, and where the binary32 clock cannot tell, a fixed-point clock
 // (kTauOne = 1 day): E to 2^-38 from a table of 128 reciprocals and a quartic series in
@@ -738,7 +741,7 @@ __device__ __forceinline__ int32_t ssa_warp_day_spec(const DevParams& p, uint64_
         break;
       }
       q = valid ? rcp_approx(a0) : 0.0f;
-      float sc = fminf(__fmul_rn(Ef, q), 4.0f);
+      float sc = __fmul_rn(Ef, q);
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const float y = __shfl_up_sync(full, sc, o);
@@ -746,7 +749,7 @@ __device__ __forceinline__ int32_t ssa_warp_day_spec(const DevParams& p, uint64_
       }
       const float d = __fadd_rn(d0, sc);
       const unsigned notcont = __ballot_sync(full, !(a0 >= 2.44140625e-4f && d <= -margin));
-      const unsigned sures = __ballot_sync(full, !valid || d >= margin);
+      const unsigned sures = __ballot_sync(full, !valid || d >= __fmaf_rn(q, 7.2759576e-12f, margin));   // 2^-37
       e = notcont ? __ffs(notcont) - 1 : 32;
       const unsigned diff = __ballot_sync(full, nc != ch) & (e < 32 ? ((1u << e) - 1u) : full);
       ch = nc;
