@@ -142,10 +142,11 @@ __device__ __noinline__ uint32_t ssa_node_day_exact(const DevParams& p, uint64_t
 // binary32 helpers of the speculative methods below.
 
 __device__ __forceinline__ float trunc_to_f32(double x) {
-  // positive normal double within float range -> float with the top 23 fraction bits
+  // positive normal double within float range -> float with the top 23 fraction bits;
+  // 0 for one that is not positive (rates are non-negative, but may be -0.0)
   const uint64_t b = double_bits(x);
   const int e = (int)(b >> 52) - 1023 + 127;
-  if (b == 0ull) return 0.0f;
+  if (!pos(x)) return 0.0f;
   return __int_as_float((int)(((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7FFFFFull)));
 }
 
@@ -626,11 +627,11 @@ __device__ __forceinline__ uint64_t neglog_q43(uint64_t j) {
   return (uint64_t)(e > 0 ? e : 0);
 }
 
-// floor(c 2^s) of a non-negative binary64 c < 2^(62-s).
+// floor(c 2^s) of a binary64 c < 2^(62-s); 0 for one that is not positive (-0.0).
 __device__ __forceinline__ uint64_t rate_fixed(double c, int s) {
+  if (!pos(c)) return 0ull;
   const uint64_t b = double_bits(c);
-  const int e = (int)(b >> 52);
-  if (e == 0) return 0ull;                          // 0 (spec_constants rules out subnormal constants)
+  const int e = (int)(b >> 52);                     // above 0: spec_constants rules out subnormal constants
   const uint64_t m = (b & ((1ull << 52) - 1)) | (1ull << 52);
   const int sh = s + e - 1023 - 52;
   return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> (-sh)) : 0ull);
@@ -670,7 +671,8 @@ __device__ __forceinline__ int32_t ssa_warp_day_spec(const DevParams& p, uint64_
     for (int j = 0; j < NA; ++j) {
       cinf[j] = __dmul_rn(p.ups[j], phi);
       herd += s.x[2 * j] + s.x[2 * j + 1];
-      top = max(top, max((int)(double_bits(cinf[j]) >> 52), (int)(double_bits(p.gam[j]) >> 52)) - 1022);   // < 2^top
+      if (pos(cinf[j])) top = max(top, (int)(double_bits(cinf[j]) >> 52) - 1022);                          // < 2^top
+      if (pos(p.gam[j])) top = max(top, (int)(double_bits(p.gam[j]) >> 52) - 1022);
     }
     if (!spec_constants<NA>(p, cinf, s.x, cinff, gamf)) return -1;
     sq = 62 - max(top, -100) - (32 - __clz(herd));   // the rates' sum stays below 2^62 units
