@@ -242,11 +242,13 @@ constexpr int kGenSmall = 4;                         // event step: compartments
 // rule decides that draw; a clock decision inside the margin hands the node-day
 // back to the binary64 method.  The results are the specification's, bit for bit.
 // A positive constant below 2^-100 (a variable that decayed for years) is taken as
-// 2^-100: its rate, at most 2^-56, is then too large by less than u / 4 of any a0~ from
-// 2^-30 on, and below that no draw is a certain continue while a certain stop only
-// becomes more certain with the true, smaller a0.
+// 2^-100: its rate is then too large by at most 2^-56, all of them by 2^-51.  For the
+// clock that is at most 2u of any a0~ from 2^-28 on (one clamped rate: u / 16); below that
+// no draw is a certain continue, while a certain stop only becomes more certain with the
+// true, smaller a0.  For a selection it is an absolute error of 2^-51 in every threshold
+// and in r~, so a selection is decisive only from 2^-49 on, besides the relative bound.
 constexpr uint32_t kGenSpecMaxSteps = 1u << 18;
-constexpr float kGenSmallA0 = 9.313226e-10f;                  // 2^-30
+constexpr float kGenSmallA0 = 3.7252903e-9f;                  // 2^-28
 constexpr float kGenBigCount = 4194304.0f;                    // 2^22
 
 // binary32 constant k_j y_q of a transition; false when outside the bounds above.
@@ -332,8 +334,8 @@ __device__ __forceinline__ float gen_sums_f32(const GenSsaArgs& a, const float (
 }
 
 // The transition r = a0 u2 fires: the number of thresholds below r (zero-width
-// intervals, from zero rates, are skipped), -1 unless r~ (within (nt + 26)u) is at
-// least 2^-17 r~ = 128u from every threshold: more than 2 nt + 34 <= 98.
+// intervals, from zero rates, are skipped), -1 unless r~ (within (nt + 26)u and 2^-51) is
+// at least 2^-17 r~ + 2^-49 from every threshold: 2^-17 = 128u, more than 2 nt + 34 <= 98.
 template <int L>
 __device__ __forceinline__ int gen_select_f32(int nt, const float (&P)[L], float r) {
   float gap = r;
@@ -345,7 +347,7 @@ __device__ __forceinline__ int gen_select_f32(int nt, const float (&P)[L], float
       gap = fminf(gap, fabsf(e));
       n += e > 0.0f ? 1 : 0;
     }
-  return gap < __fmul_rn(r, 7.6293945e-6f) || n >= nt ? -1 : n;
+  return gap < __fmaf_rn(r, 7.6293945e-6f, 1.7763568e-15f) || n >= nt ? -1 : n;
 }
 
 // The thread method: one node per thread.  A firing n applies chg[n] = two (row,
@@ -493,7 +495,8 @@ __device__ __forceinline__ int32_t gen_draws_node_day(const GenSsaArgs& a, const
       int next = -1;
       if (valid) {
         next = gen_select_f32<L>(nt, P, __fmul_rn(a0, u2f));
-        if (next < 0) {
+        // (a draw that cannot be a certain continue ends the day: its choice is not needed)
+        if (next < 0 && (EXACT || a0 >= kGenSmallA0)) {
           column_to_int(xf, m.nc);
           next = gen_exact_choice(m, p, reinterpret_cast<const int32_t*>(xf), kGenThreads, y, uniform_open(w.z, w.w));
           column_to_float(xf, m.nc);
