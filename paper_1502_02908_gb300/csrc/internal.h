@@ -220,12 +220,12 @@ cudaError_t launch_pack_touched(const int32_t* counts, const int32_t* touched, i
 cudaError_t launch_unpack_touched(int32_t* counts, const int32_t* touched, int n_t, int N, int64_t planes,
                                   const int32_t* in, const int32_t* bounds, int world, const int32_t* ids,
                                   cudaStream_t st);
-// Storage order of `planes` planes of N elements of `size` (4 or 8) bytes: to node order
-// (out[ids[i]] = in[i]) or from it (out[i] = in[ids[i]]).
-cudaError_t launch_to_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
-                            cudaStream_t st);
-cudaError_t launch_from_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
-                              cudaStream_t st);
+// Storage order of pc planes of N counts and pf planes of phi: to node order (out[ids[i]] =
+// in[i]) or from it (out[i] = in[ids[i]]).
+cudaError_t launch_to_nodes(int32_t* c_out, const int32_t* c_in, int64_t pc, double* f_out, const double* f_in, int64_t pf,
+                            const int32_t* ids, int N, cudaStream_t st);
+cudaError_t launch_from_nodes(int32_t* c_out, const int32_t* c_in, int64_t pc, double* f_out, const double* f_in, int64_t pf,
+                              const int32_t* ids, int N, cudaStream_t st);
 cudaError_t launch_debug_neglog(const uint64_t* j, double* out, int64_t n, cudaStream_t st);
 cudaError_t launch_debug_neglog_f32(const uint64_t* j, float* out, int64_t n, cudaStream_t st);
 

@@ -11,6 +11,8 @@
 // over the touched herds rather than over a split of the event list.
 #include "internal.h"
 
+#include <algorithm>
+
 namespace episim {
 namespace {
 
@@ -48,16 +50,19 @@ __global__ void __launch_bounds__(256) k_unpack_touched(int32_t* __restrict__ co
   }
 }
 
-// Storage order to node order and back, plane by plane; the scattered side is one
-// plane's (a few hundred KB: in L2), the other streams.
-template <class T, bool TO_NODES>
-__global__ void __launch_bounds__(256) k_reorder(T* __restrict__ out, const T* __restrict__ in,
-                                                  const int32_t* __restrict__ ids, int N, int64_t planes) {
-  const int64_t total = planes * N;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t base = i / N * N;
-    const int64_t node = base + ids[i - base];
-    if (TO_NODES) out[node] = in[i]; else out[i] = in[node];
+// Storage order to node order and back: a thread takes one position through the planes
+// (grid y of them at a time), so its node is read once.  The scattered side of a plane (a
+// few hundred KB) stays in L2, the other streams.
+template <bool TO_NODES>
+__global__ void __launch_bounds__(256) k_reorder(int32_t* __restrict__ c_out, const int32_t* __restrict__ c_in, int64_t pc,
+                                                  double* __restrict__ f_out, const double* __restrict__ f_in, int64_t pf,
+                                                  const int32_t* __restrict__ ids, int N) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int64_t id = ids[i], to = TO_NODES ? id : i, from = TO_NODES ? i : id;
+  for (int64_t p = blockIdx.y; p < pc + pf; p += gridDim.y) {
+    if (p < pc) c_out[p * N + to] = c_in[p * N + from];
+    else f_out[(p - pc) * N + to] = f_in[(p - pc) * N + from];
   }
 }
 
@@ -67,24 +72,24 @@ unsigned grid_for(int64_t total) {
 }
 
 template <bool TO_NODES>
-cudaError_t launch_reorder(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
-                           cudaStream_t st) {
-  if (N <= 0 || planes <= 0) return cudaSuccess;
-  if (size == 8) k_reorder<double, TO_NODES><<<grid_for(planes * N), 256, 0, st>>>((double*)out, (const double*)in, ids, N, planes);
-  else k_reorder<int32_t, TO_NODES><<<grid_for(planes * N), 256, 0, st>>>((int32_t*)out, (const int32_t*)in, ids, N, planes);
+cudaError_t launch_reorder(int32_t* c_out, const int32_t* c_in, int64_t pc, double* f_out, const double* f_in, int64_t pf,
+                           const int32_t* ids, int N, cudaStream_t st) {
+  if (N <= 0 || pc + pf <= 0) return cudaSuccess;
+  const dim3 grid((unsigned)((N + 255) / 256), (unsigned)std::min<int64_t>(pc + pf, 64));
+  k_reorder<TO_NODES><<<grid, 256, 0, st>>>(c_out, c_in, pc, f_out, f_in, pf, ids, N);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_to_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
-                            cudaStream_t st) {
-  return launch_reorder<true>(out, in, ids, N, planes, size, st);
+cudaError_t launch_to_nodes(int32_t* c_out, const int32_t* c_in, int64_t pc, double* f_out, const double* f_in, int64_t pf,
+                            const int32_t* ids, int N, cudaStream_t st) {
+  return launch_reorder<true>(c_out, c_in, pc, f_out, f_in, pf, ids, N, st);
 }
 
-cudaError_t launch_from_nodes(void* out, const void* in, const int32_t* ids, int N, int64_t planes, int size,
-                              cudaStream_t st) {
-  return launch_reorder<false>(out, in, ids, N, planes, size, st);
+cudaError_t launch_from_nodes(int32_t* c_out, const int32_t* c_in, int64_t pc, double* f_out, const double* f_in, int64_t pf,
+                              const int32_t* ids, int N, cudaStream_t st) {
+  return launch_reorder<false>(c_out, c_in, pc, f_out, f_in, pf, ids, N, st);
 }
 
 cudaError_t launch_pack_touched(const int32_t* counts, const int32_t* touched, int n_t, int N, int64_t planes,
