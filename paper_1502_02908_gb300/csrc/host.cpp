@@ -338,6 +338,24 @@ cudaError_t alloc_staging(sim_handle* h) {
   return e;
 }
 
+// Initial herd of every node (at most 2^30), and the nodes [lo, hi) by it, largest first,
+// ties by node.
+std::vector<int64_t> herds(const sim_handle* h) {
+  const int N = h->cfg.n_nodes;
+  std::vector<int64_t> herd((size_t)N, 0);
+  for (int c = 0; c < h->nc; ++c)
+    for (int v = 0; v < N; ++v) herd[(size_t)v] += h->u0[(size_t)c * N + v];
+  return herd;
+}
+std::vector<int32_t> by_herd(const std::vector<int64_t>& herd, int32_t lo, int32_t hi) {
+  std::vector<uint64_t> key((size_t)(hi - lo));
+  for (int32_t v = lo; v < hi; ++v) key[(size_t)(v - lo)] = (uint64_t)((1ll << 30) - herd[(size_t)v]) << 32 | (uint32_t)v;
+  std::sort(key.begin(), key.end());
+  std::vector<int32_t> nodes(key.size());
+  for (size_t i = 0; i < key.size(); ++i) nodes[i] = (int32_t)(uint32_t)key[i];
+  return nodes;
+}
+
 size_t n_counts(const sim_handle* h) { return (size_t)h->cfg.n_replicates * h->nc * h->cfg.n_nodes; }
 size_t n_phi(const sim_handle* h) { return (size_t)h->cfg.n_replicates * h->cfg.n_nodes; }
 
@@ -470,8 +488,11 @@ sim_status build_split(sim_handle* h) {
 // upsilon phi (1 - p) = gamma p gives p = 1 - beta gamma / (upsilon alpha) up to eps.
 double endemic_rate(const sim_handle* h) {
   double class_animals[kMaxAge] = {0.0, 0.0, 0.0}, total = 0.0, phi0 = 0.0, sum = 0.0;
-  for (int c = 0; c < h->nc; ++c)
-    for (int v = 0; v < h->cfg.n_nodes; ++v) class_animals[c / 2] += h->u0[(size_t)c * h->cfg.n_nodes + v];
+  for (int c = 0; c < h->nc; ++c) {
+    int64_t n = 0;
+    for (int v = 0; v < h->cfg.n_nodes; ++v) n += h->u0[(size_t)c * h->cfg.n_nodes + v];
+    class_animals[c / 2] += (double)n;
+  }
   for (double c : class_animals) total += c;
   if (total <= 0.0) return 0.0;
   for (double p : h->phi0) phi0 += p;
@@ -525,13 +546,19 @@ int32_t auto_threshold(const sim_handle* h) {
 // each (similar work per warp).  threshold < 0: automatic (above).
 sim_status set_order(sim_handle* h, int32_t threshold) {
   const int N = h->cfg.n_nodes;
-  std::vector<int64_t> herd(N, 0);
-  for (int c = 0; c < h->nc; ++c)
-    for (int v = 0; v < N; ++v) herd[v] += h->u0[(size_t)c * N + v];
+  const std::vector<int64_t> herd = herds(h);
   const int n_own = h->node_hi - h->node_lo;
-  std::vector<int32_t> order(n_own);
-  for (int i = 0; i < n_own; ++i) order[i] = h->node_lo + i;
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return herd[a] > herd[b]; });
+  std::vector<int32_t> order;
+  if (h->pos.empty()) {
+    order = by_herd(herd, h->node_lo, h->node_hi);
+  } else {                          // the storage order is that sort of every node
+    order.resize((size_t)n_own);
+    std::vector<int32_t> ids((size_t)N);
+    for (int v = 0; v < N; ++v) ids[(size_t)h->pos[(size_t)v]] = v;
+    int i = 0;
+    for (int32_t v : ids)
+      if (v >= h->node_lo && v < h->node_hi) order[(size_t)i++] = v;
+  }
   h->herd_sorted.resize((size_t)n_own);
   for (int i = 0; i < n_own; ++i) h->herd_sorted[(size_t)i] = (int32_t)herd[(size_t)order[(size_t)i]];   // <= 2^30
   h->animal_rate = endemic_rate(h);
@@ -1231,12 +1258,7 @@ sim_status create_impl(const sim_config* cfg, const int32_t* u0, const double* p
   // (whose sums run over the nodes in order) the nodes stay as they are.
   if (!dev_counts && !(h->cfg.flags & SIM_FLAG_SCORE) && (int64_t)N * R >= ((int64_t)1 << 15)) {
     try {
-      std::vector<int64_t> herd((size_t)N, 0);
-      for (int c = 0; c < h->nc; ++c)
-        for (int v = 0; v < N; ++v) herd[(size_t)v] += h->u0[(size_t)c * N + v];
-      std::vector<int32_t> ids((size_t)N);
-      for (int v = 0; v < N; ++v) ids[(size_t)v] = v;
-      std::stable_sort(ids.begin(), ids.end(), [&](int32_t a, int32_t b) { return herd[(size_t)a] > herd[(size_t)b]; });
+      const std::vector<int32_t> ids = by_herd(herds(h), 0, N);
       h->pos.resize((size_t)N);
       for (int i = 0; i < N; ++i) h->pos[(size_t)ids[(size_t)i]] = i;
       if (e == cudaSuccess) e = dalloc(&h->d_ids, (size_t)N);
