@@ -1187,6 +1187,10 @@ __device__ __forceinline__ void node_day_work(const SsaArgs& a, int r, int v, bo
       }
     } else {
       if (role == kRoleGroup) {                    // every lane of the warp takes part
+        // a unit with fewer than four nodes comes here in two parts, and without this every
+        // collective of the method runs twice over: 1,000 herds, one such unit, 200 days on
+        // one GB300, 31 us a launch against 15
+        __syncwarp();
         f = a.clock_margin ? ssa_seg_node_day<NA, kGroupLanes>(p, a.seed, rep, id, a.day, phi, a.clock_margin,
                                                                active, s)
                            : (active ? -1 : 0);
