@@ -310,8 +310,8 @@ sim_status sim_schedule_events(int32_t n_nodes, int32_t model, int32_t max_days,
  * and time 32 steps at once; suited to herds with many transitions per day);
  * the others one per thread.  -1 = automatic (the largest herds, as many as leave
  * each unit of work -- a herd per warp, 32 herds per warp -- a resident warp, and
- * herds whose one-thread day would outlast the whole step); a very large value
- * disables the warp path.  Results do not depend on this setting.  Score
+ * herds whose one-thread day would outlast the whole step; every herd with
+ * SIM_OPT_CLOCK_MARGIN 0); a very large value disables the warp path.  Results do not depend on this setting.  Score
  * mode always uses one thread per node.  Synchronises the device. */
 sim_status sim_tune(sim_handle* h, int32_t warp_herd_threshold);
 /* Number of nodes currently simulated one per warp (-1 for a NULL handle). */
