@@ -245,6 +245,7 @@ sim_status latched(gen_handle* h) {
 constexpr int32_t kGenMaxMargin = 16;
 constexpr int64_t kAutoWarpThreshold = 600;
 constexpr int64_t kAutoGroupThreshold = 300;
+constexpr int64_t kAutoGroupExact = 150;            // without the binary32 methods
 
 // Warp and group nodes of the node order.  Automatic warp nodes: as many of the largest
 // as let every unit (a node per warp, then 32 nodes per warp) have a resident warp of its
@@ -254,15 +255,24 @@ constexpr int64_t kAutoGroupThreshold = 300;
 // warp nodes (one wave), 16.5 with 407, 20.6 with 4,316 (two waves); Erlang on 1,500 nodes
 // x 40 days 3.3 ms with every node a warp node, 8.1 with none.  Automatic group nodes: 300
 // animals or more (24 us a day for herds of 150-300 against 27 us one per thread).
+// Without the binary32 methods (margin 0) a warp node costs more and a thread node's day
+// grows faster: one wave of warps only where it holds every node, and groups from 150 on
+// while the nodes fit one wave of threads (SEIRS on 37,000 nodes x 60 days 6.5 ms, 8.4 with
+// one wave of warp nodes and groups from 300; SISe3 3.5 and 4.5, ten replicates x 20 days
+// 6.5 and 4.6; Erlang, every node a warp's, 9.4 ms, 13.5 without).
 void set_n_big(gen_handle* h) {
   const int64_t N = (int64_t)h->pop_sorted.size(), R = h->cfg.n_replicates;
   const int64_t thr = h->warp_threshold < 0 ? kAutoWarpThreshold : h->warp_threshold;
-  const int64_t gthr = h->group_threshold < 0 ? kAutoGroupThreshold : h->group_threshold;
+  const bool exact = h->clock_margin_log2 == 0;
+  const bool one_wave = N * R <= (int64_t)h->ssa.resident_blocks * kGenThreads;
+  const int64_t gthr = h->group_threshold >= 0 ? h->group_threshold
+                                               : (exact && one_wave ? kAutoGroupExact : kAutoGroupThreshold);
   int64_t n = 0;
   if (h->warp_threshold < 0) {
     // largest n with n + (N - n) / 32 <= per
     const int64_t per = (int64_t)h->ssa.resident_blocks * (kGenThreads / 32) * 9 / 10 / R;
     n = std::min(N, std::max<int64_t>(0, (32 * per - N) / 31));
+    if (exact && one_wave && n < N) n = 0;
   }
   while (n < N && h->pop_sorted[n] >= thr) ++n;
   int64_t g = n;
@@ -648,6 +658,7 @@ sim_status gen_set_option(gen_handle* h, int32_t option, int64_t value) {
     if (value < 0 || value > 16) return gfail(h, SIM_E_INVALID_ARG, "clock margin exponent %lld outside [0, 16]", (long long)value);
     free_graph(h);
     h->clock_margin_log2 = (int32_t)value;
+    set_n_big(h);
     return SIM_OK;
   }
   return gfail(h, SIM_E_INVALID_ARG, "option %d unknown", option);
