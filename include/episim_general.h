@@ -166,12 +166,12 @@ sim_status gen_counters(gen_handle* h, int64_t* counters);
  *   GEN_OPT_WARP_THRESHOLD: nodes whose initial population (sum of u0) is at least
  *       this run the stochastic step one per warp, 32 draws at a time with a
  *       fixed-point iteration over the lanes (-1: automatic, the largest nodes, as
- *       many as leave each unit of work a resident warp, and those from 600 on; with
- *       margin 0 the first only where that is every node);
+ *       many as leave each unit of work a resident warp, and those from 600 on; where
+ *       every node-day runs exactly, the first only where that is every node);
  *   GEN_OPT_GROUP_THRESHOLD: nodes below the warp threshold whose initial
  *       population is at least this run four per warp, 8 lanes and 8 draws at a
- *       time each (-1: automatic, 300, or 150 with margin 0 while the nodes fit one
- *       wave of threads); the rest one per thread;
+ *       time each (-1: automatic, 300, or 150 where every node-day runs exactly
+ *       and the nodes fit one wave of threads); the rest one per thread;
  *   GEN_OPT_CLOCK_MARGIN: k in [0, 16].  Every node-day (one per thread, per
  *       warp or per 8-lane segment) first runs with binary32 rates and partial
  *       sums and a binary32 clock whose distance to the binary64 clock of Eq.
@@ -182,7 +182,8 @@ sim_status gen_counters(gen_handle* h, int64_t* counters);
  *       within the margin of the day's end reruns the node-day with the binary64
  *       arithmetic.  k = 16 (default) is the method's own bound, below 2^-16;
  *       smaller k, a margin of 2^-k, only reruns more node-days; 0 runs every
- *       node-day exactly. */
+ *       node-day exactly, and so does k <= 7 with both thresholds automatic where
+ *       not every node is a warp node. */
 enum { GEN_OPT_LAUNCH = 1, GEN_OPT_WARP_THRESHOLD = 2, GEN_OPT_GROUP_THRESHOLD = 3, GEN_OPT_CLOCK_MARGIN = 4 };
 sim_status gen_set_option(gen_handle* h, int32_t option, int64_t value);
 

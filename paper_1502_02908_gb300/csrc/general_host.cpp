@@ -43,6 +43,7 @@ struct gen_handle {
   std::vector<int64_t> pop_sorted;  // initial node populations in the node order (descending)
   int32_t warp_threshold = -1;      // initial population from which a node gets a warp (-1: automatic)
   int32_t clock_margin_log2 = 16;   // binary32 clock margin 2^-k (0: exact only)
+  bool exact = false;               // binary64 methods only (set_n_big)
   int32_t group_threshold = -1;     // ... an 8-lane segment (-1: automatic)
   int32_t n_big = 0;                // nodes simulated one per warp
   int32_t n_mid = 0;                // nodes simulated four per warp
@@ -246,6 +247,7 @@ constexpr int32_t kGenMaxMargin = 16;
 constexpr int64_t kAutoWarpThreshold = 600;
 constexpr int64_t kAutoGroupThreshold = 300;
 constexpr int64_t kAutoGroupExact = 150;            // without the binary32 methods
+constexpr int32_t kExactMargin = 7;                 // margin exponents up to here may do without them
 
 // Warp and group nodes of the node order.  Automatic warp nodes: as many of the largest
 // as let every unit (a node per warp, then 32 nodes per warp) have a resident warp of its
@@ -260,20 +262,25 @@ constexpr int64_t kAutoGroupExact = 150;            // without the binary32 meth
 // while the nodes fit one wave of threads (SEIRS on 37,000 nodes x 60 days 6.5 ms, 8.4 with
 // one wave of warp nodes and groups from 300; SISe3 3.5 and 4.5, ten replicates x 20 days
 // 6.5 and 4.6; Erlang, every node a warp's, 9.4 ms, 13.5 without).
+// A margin so wide that a good part of the node-days is run again (2^-7 and wider) goes to
+// the binary64 methods outright where nodes share warps, since a warp reruns its nodes one
+// after the other (both thresholds automatic; chosen ones keep the binary32 methods):
+// SISe3 on 37,000 nodes x 60 days 3.5 ms, with reruns 4.9 at 2^-6 and 18.8 at 2^-1.
 void set_n_big(gen_handle* h) {
   const int64_t N = (int64_t)h->pop_sorted.size(), R = h->cfg.n_replicates;
-  const int64_t thr = h->warp_threshold < 0 ? kAutoWarpThreshold : h->warp_threshold;
-  const bool exact = h->clock_margin_log2 == 0;
-  const bool one_wave = N * R <= (int64_t)h->ssa.resident_blocks * kGenThreads;
-  const int64_t gthr = h->group_threshold >= 0 ? h->group_threshold
-                                               : (exact && one_wave ? kAutoGroupExact : kAutoGroupThreshold);
   int64_t n = 0;
   if (h->warp_threshold < 0) {
     // largest n with n + (N - n) / 32 <= per
     const int64_t per = (int64_t)h->ssa.resident_blocks * (kGenThreads / 32) * 9 / 10 / R;
     n = std::min(N, std::max<int64_t>(0, (32 * per - N) / 31));
-    if (exact && one_wave && n < N) n = 0;
   }
+  h->exact = h->clock_margin_log2 == 0 ||
+             (h->clock_margin_log2 <= kExactMargin && h->warp_threshold < 0 && h->group_threshold < 0 && n < N);
+  const bool one_wave = N * R <= (int64_t)h->ssa.resident_blocks * kGenThreads;
+  if (h->exact && one_wave && n < N) n = 0;
+  const int64_t thr = h->warp_threshold < 0 ? kAutoWarpThreshold : h->warp_threshold;
+  const int64_t gthr = h->group_threshold >= 0 ? h->group_threshold
+                                               : (h->exact && one_wave ? kAutoGroupExact : kAutoGroupThreshold);
   while (n < N && h->pop_sorted[n] >= thr) ++n;
   int64_t g = n;
   while (g < N && h->pop_sorted[g] >= gthr) ++g;
@@ -289,7 +296,7 @@ sim_status enqueue_days(gen_handle* h, int32_t d0, int32_t nd, cudaStream_t st) 
     s.order = h->d_order; s.ctr = h->d_ctr; s.seed = h->cfg.seed; s.rep_base = h->cfg.replicate_base;
     s.N = N; s.R = R; s.day = d; s.n_big = h->n_big; s.n_mid = h->n_mid;
     s.prologue = (d > d0 && h->ny > 0 && h->model.y_source != GEN_Y_PRE_EVENT) ? 1 : 0;
-    s.clock_margin = h->clock_margin_log2 > 0 ? (1ull << (62 - h->clock_margin_log2)) : 0ull;
+    s.clock_margin = h->exact ? 0ull : (1ull << (62 - h->clock_margin_log2));
     // the binary32 methods' own bound, (nt + 44) 2^-24, is below 2^-16: that is the
     // margin at the default exponent; a wider margin is taken as asked
     s.margin_f = h->clock_margin_log2 >= kGenMaxMargin ? std::ldexp((float)(h->nt + 44), -24)
