@@ -395,7 +395,7 @@ def batched_leg(args, B, W, torch, plain_value, hbm_peak, fp64, oracle_check):
     trans = int((c1[:, 0] - c0[:, 0]).sum()) // (warm + steps)
     evs = int((c1[:, 1] - c0[:, 1]).sum()) // (warm + steps)
     sim.close()
-    B.batch_shape(*B.BATCH_SHAPES[0])
+    B.batch_shape_auto()
     line = {"workload": f"SISe3 national network, {w.R} replicates x {w.T} days, own (upsilon, gamma) each",
             "value": value, "unit": "node-days/s", "steps": steps, "warmup": warm, "ms_per_step": ms,
             "events_per_s": (trans + evs) / (ms / 1000), "transitions_per_s": trans / (ms / 1000),

@@ -402,19 +402,22 @@ sim_status sim_run_batch(sim_handle** handles, int32_t n, const int32_t* until, 
 
 /* Block shape of sim_run_batch's persistent kernel (and of SIM_LAUNCH_PERSISTENT)
  * for the calls that follow, process-wide: `threads` threads a block and
- * `blocks_per_sm` resident blocks an SM, one of 256 x 2 (the default), 256 x 1
- * and 128 x 4.  A stochastic-step chunk is one block's worth of nodes, one a
+ * `blocks_per_sm` resident blocks an SM, one of 256 x 2, 256 x 1 and 128 x 4.  A stochastic-step chunk is one block's worth of nodes, one a
  * thread (or of herds on the warp path, one a warp).  The blocks of an SM share
  * 220 KB of shared memory for the staged event step: a day whose staged step
  * needs more than 220 KB / blocks_per_sm runs the global-memory variant.  More
  * resident blocks hide more of the stochastic step's latency at a register budget
  * of 65,536 / (threads x blocks_per_sm) a thread.  Results do not depend on the
- * shape (every random number is keyed by node, day and event position).  With the
- * default shape a run whose per-thread nodes would not fill its blocks takes one block
- * an SM.  The
- * paper has no counterpart: this is a launch-tuning knob.  Errors:
- * SIM_E_INVALID_ARG for any other shape. */
+ * shape (every random number is keyed by node, day and event position).  A shape
+ * that is set holds for every later call, until sim_batch_shape_auto leaves the
+ * choice to the library again, as it is at first: 256 x 2, or 256 x 1 for runs
+ * whose nodes would not fill two blocks an SM.  The paper has no counterpart: this
+ * is a launch-tuning knob.  Errors: SIM_E_INVALID_ARG for any other shape. */
 sim_status sim_batch_shape(int32_t threads, int32_t blocks_per_sm);
+sim_status sim_batch_shape_auto(void);
+/* The shape that a run of that many blocks' worth of nodes (256 each, summed over
+ * instances and replicates) takes on a device of `sms` SMs (host only). */
+sim_status sim_debug_batch_shape(int64_t blocks_worth, int32_t sms, int32_t* threads, int32_t* blocks_per_sm);
 
 /* Test hook for the dataflow loop's failure path: runs ndays days from the
  * current day (>= 1) with SIM_LAUNCH_FLOW, but with the first stochastic-step

@@ -44,16 +44,18 @@ def apply(sim, best):
     sim.set_launch(best["launch"])
     if best.get("batch_shape"):
         B.batch_shape(*best["batch_shape"])
+    elif best["launch"] == "persistent":
+        B.batch_shape_auto()
 
 
 def autotune(workload, days=None, thresholds=WARP_THRESHOLDS, modes=LAUNCH_MODES, repeats=2,
-             groups=(1 << 30,), shapes=(B.BATCH_SHAPES[0],)):
+             groups=(1 << 30,), shapes=(None,)):
     """Returns (best {"warp_threshold", "group_threshold", "launch", "batch_shape"},
     table [(threshold, group threshold, mode, batch shape, ms)]).  Group thresholds
     at or above the warp threshold are skipped (no herd would take the group path);
-    the persistent mode is timed in every block shape of `shapes` (batch_shape is
-    None for the other modes).  The library's default batch shape is restored
-    afterwards; apply() sets the winner's."""
+    the persistent mode is timed in every block shape of `shapes` (None: the
+    library's choice; batch_shape is None for the other modes).  The choice is left
+    to the library afterwards; apply() sets the winner's."""
     import torch
     w = workload
     nd = min(w.T, days if days is not None else max(10, w.T // 10))
@@ -69,6 +71,8 @@ def autotune(workload, days=None, thresholds=WARP_THRESHOLDS, modes=LAUNCH_MODES
             sim.set_launch(mode)
             if shape:
                 B.batch_shape(*shape)
+            else:
+                B.batch_shape_auto()
             best = float("inf")
             for rep in range(repeats + 1):                 # first pass warms up (graph capture, caches)
                 sim.set_state(u0, phi0, 0)
@@ -88,7 +92,7 @@ def autotune(workload, days=None, thresholds=WARP_THRESHOLDS, modes=LAUNCH_MODES
             table.append((thr, gthr, mode, shape, best))
     finally:
         sim.close()
-        B.batch_shape(*B.BATCH_SHAPES[0])
+        B.batch_shape_auto()
     thr, gthr, mode, shape, _ = min(table, key=lambda x: x[4])
     return {"warp_threshold": thr, "group_threshold": gthr, "launch": mode, "batch_shape": shape}, table
 

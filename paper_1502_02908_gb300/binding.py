@@ -116,6 +116,8 @@ def load_library(build_if_missing: bool = True):
             "sim_unpack_touched": [vp, vp, i32, pi32, vp],
             "sim_run_batch": [P(vp), i32, pi32, vp],
             "sim_batch_shape": [i32, i32],
+            "sim_batch_shape_auto": [],
+            "sim_debug_batch_shape": [i64, i32, pi32, pi32],
             "sim_set_option": [vp, i32, i64],
             "sim_set_regions": [vp, pi32, i32],
             "sim_set_params": [vp, vp],
@@ -483,7 +485,7 @@ def run_batch(sims, until=None, stream=None):
     _check(L, None, status)
 
 
-BATCH_SHAPES = ((256, 2), (256, 1), (128, 4))   # the first is the library's default
+BATCH_SHAPES = ((256, 2), (256, 1), (128, 4))
 
 
 def batch_shape(threads: int, blocks_per_sm: int):
@@ -491,6 +493,20 @@ def batch_shape(threads: int, blocks_per_sm: int):
     persistent kernel, process-wide; one of BATCH_SHAPES."""
     L = load_library()
     _check(L, None, L.sim_batch_shape(int(threads), int(blocks_per_sm)))
+
+
+def batch_shape_auto():
+    """Leaves the block shape to the library again, run by run (as it is at first)."""
+    L = load_library()
+    _check(L, None, L.sim_batch_shape_auto())
+
+
+def debug_batch_shape(blocks_worth: int, sms: int):
+    """The shape a run of that many blocks' worth of nodes takes on sms SMs."""
+    L = load_library()
+    t, b = ctypes.c_int32(0), ctypes.c_int32(0)
+    _check(L, None, L.sim_debug_batch_shape(int(blocks_worth), int(sms), ctypes.byref(t), ctypes.byref(b)))
+    return t.value, b.value
 
 
 def debug_div(x, y, out, ref, n, device):

@@ -2264,6 +2264,16 @@ namespace {
 long long g_batch_spin_limit = 5000000;   // ~2 s of polling per wait
 bool g_batch_stall = false;               // test switch, see sim_debug_batch_stall
 BatchShape g_batch_shape = BatchShape::k256x2;   // see sim_batch_shape
+bool g_batch_shape_set = false;           // by a caller: then kept for every run
+
+// Block shape of a run of `worth` blocks' worth (256) of nodes.  A caller's shape stays.
+// The library's own, two blocks of 256 threads an SM, gives way to one, with twice the
+// registers a thread and fewer blocks polling, for runs that would not fill them (32
+// uneven instances: 54 ms a run against 73).
+BatchShape run_batch_shape(int64_t worth, int sms) {
+  if (!g_batch_shape_set && worth <= 2LL * sms) return BatchShape::k256x1;
+  return g_batch_shape;
+}
 }
 
 sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void* stream) {
@@ -2294,15 +2304,9 @@ sim_status sim_run_batch(sim_handle** hs, int32_t n, const int32_t* until, void*
   std::vector<long long> cumA(ni + 1, 0), cumB(ni + 1, 0), cumF(ni + 1, 0);
   long long n_counters = 0;
   int smem_cap = 0;
-  // The default shape gives way to one block an SM, with twice the registers a thread and
-  // fewer blocks polling, for runs whose per-thread nodes would not fill its blocks (32
-  // uneven instances: 54 ms a run against 73).
-  BatchShape shape = g_batch_shape;
-  {
-    long long nodes = 0;
-    for (int k = 0; k < ni; ++k) nodes += (long long)hs[idx[k]]->cfg.n_replicates * ((hs[idx[k]]->cfg.n_nodes + 255) / 256);
-    if (shape == BatchShape::k256x2 && nodes <= 2LL * hs[idx[0]]->sm_count) shape = BatchShape::k256x1;
-  }
+  long long nodes = 0;
+  for (int k = 0; k < ni; ++k) nodes += (long long)hs[idx[k]]->cfg.n_replicates * ((hs[idx[k]]->cfg.n_nodes + 255) / 256);
+  const BatchShape shape = run_batch_shape(nodes, hs[idx[0]]->sm_count);
   const int threads = batch_threads(shape);
   // two blocks an SM share its 228 KB of shared memory; a day whose staged event
   // step needs more takes the global-memory variant
@@ -2473,6 +2477,21 @@ sim_status sim_batch_shape(int32_t threads, int32_t blocks_per_sm) {
   else if (threads == 128 && blocks_per_sm == 4) g_batch_shape = BatchShape::k128x4;
   else return fail(nullptr, SIM_E_INVALID_ARG, "batch shape %d x %d is not one of 256x1, 256x2, 128x4",
                    threads, blocks_per_sm);
+  g_batch_shape_set = true;
+  return SIM_OK;
+}
+
+sim_status sim_batch_shape_auto(void) {
+  g_batch_shape = BatchShape::k256x2;
+  g_batch_shape_set = false;
+  return SIM_OK;
+}
+
+sim_status sim_debug_batch_shape(int64_t blocks_worth, int32_t sms, int32_t* threads, int32_t* blocks_per_sm) {
+  if (blocks_worth < 0 || sms < 1 || !threads || !blocks_per_sm) return SIM_E_INVALID_ARG;
+  const BatchShape s = run_batch_shape(blocks_worth, sms);
+  *threads = batch_threads(s);
+  *blocks_per_sm = batch_min_blocks(s);
   return SIM_OK;
 }
 

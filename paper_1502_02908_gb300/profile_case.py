@@ -30,7 +30,7 @@ def main(argv=None):
     ap.add_argument("--launch", choices=["stream", "flow", "persistent"], default="stream",
                     help="stream: one launch per kernel and day; flow: one dataflow launch for all days; "
                          "persistent: one persistent batch launch")
-    ap.add_argument("--shape", default="256x2", help="persistent batch block shape, threads x blocks an SM")
+    ap.add_argument("--shape", help="persistent batch block shape, threads x blocks an SM (default: the library's choice)")
     ap.add_argument("--instances", type=int, default=64, help="uneven: how many of the 512 instances")
     args = ap.parse_args(argv)
     import torch
@@ -38,7 +38,8 @@ def main(argv=None):
     from . import workloads as W
     from .build import build
     build()
-    B.batch_shape(*(int(x) for x in args.shape.split("x")))
+    if args.shape:
+        B.batch_shape(*(int(x) for x in args.shape.split("x")))
     if args.case == "uneven":
         ws = W.uneven_batch()[:args.instances]
         sims = [B.Sim.from_workload(w) for w in ws]
