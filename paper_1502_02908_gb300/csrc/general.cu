@@ -581,7 +581,7 @@ __device__ __forceinline__ int32_t gen_draws_node_day(const GenSsaArgs& a, const
 // block of 128 nodes each): SIR 2,000 nodes x 60 days 2.0 -> 1.2 ms, Erlang 1,500 x 40
 // 13.8 -> 3.3 ms, SEIRS midpoint 37,000 x 365 26.1 -> 16.4 ms, SISe3 37,000 x 365
 // 20.1 -> 13.5 ms; with the byte sums, overlapped starts and a kept graph since then
-// 0.91, 2.8, 14.0 and 11.0-13.4 ms.
+// 0.91, 2.8, 14.0 and 11.0-13.4 ms (SIR 0.77 and SEIRS 13.0 with k_gen_events_small).
 //
 // The stochastic step: warps of a resident grid (as node_day_dealt deals its units) take
 // the warp nodes first (largest first, a node's replicates together), then units of four

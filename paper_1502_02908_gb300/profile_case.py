@@ -8,14 +8,14 @@ captures day D's stochastic step).
     python -m paper_1502_02908_gb300.profile_case batched --days 30 --launch persistent
     python -m paper_1502_02908_gb300.profile_case uneven --instances 64
 
-Cases: ``national`` (SISe3, 37,000 herds, 3M events; warp path from 800
-animals, group path from 200, the bench's tuned shape), ``batched`` (the national
-network with 256 replicates, every herd on the per-thread path), ``general``
-(SISe3 written in the general model), ``uneven`` (the first `--instances` of the
+Cases: ``national`` (SISe3, 37,000 herds, 3M events), ``batched`` (the national
+network with 256 replicates), ``general`` (SISe3 written in the general model), all
+with the automatic thresholds, ``uneven`` (the first `--instances` of the
 512-instance uneven batch, whole horizons, in one persistent launch).  Launches go
 to the stream one by one (no CUDA graph), so each kernel launch is capturable;
 with ``--launch flow`` the days run as one dataflow launch, with ``--launch
-persistent`` as one persistent batch launch (block shape ``--shape``).
+persistent`` as one persistent batch launch (block shape ``--shape``, else the
+library's choice).
 """
 from __future__ import annotations
 
@@ -53,18 +53,10 @@ def main(argv=None):
         w = W.as_general(W.sise3_national())
         w.T = min(args.days, w.T)
         s = B.GenSim.from_workload(w)
-        s.set_warp_threshold(600)
-        s.set_group_threshold(300)
     else:
         w = W.sise3_national() if args.case == "national" else W.sise3_batched(R=256, T=365)
         w.T = min(args.days, w.T)
         s = B.Sim.from_workload(w)
-        if args.case == "national":
-            s.set_group_threshold(200)
-            s.tune(800)
-        else:
-            s.set_group_threshold(1 << 30)
-            s.tune(1 << 30)
     s.set_launch(args.launch if args.case != "general" else "stream")
     s.run(w.T)
     torch.cuda.synchronize()
